@@ -288,7 +288,11 @@ __global__ void __launch_bounds__(SCORE_THREADS, 2) k_score_stream(const __grid_
       khi = __vimax3_u16x2(khi, ahi.x & 0x7FFF7FFFu, ahi.y & 0x7FFF7FFFu);
       khi = __vimax3_u16x2(khi, ahi.z & 0x7FFF7FFFu, ahi.w & 0x7FFF7FFFu);
     }
-    // the stage (page and query rows) has been read: hand it back to the producer
+    // The stage (page and query rows) has been read: hand it back to the producer, whose next copy into it goes through
+    // the asynchronous proxy.  The arrive alone orders reads against accesses of the generic proxy only: without the
+    // fence a page's last 64 bytes were now and then overwritten by the stage's next page before they had been read
+    // (one step in three at 32 heads x 131,071 tokens, with the walk kernel on the same SMs).
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[stage]);
 #pragma unroll
