@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
           const int bit = __ffs(word(c)) - 1, j = j0 + c * 32 + bit;
           int ph = __shfl_sync(FULL, jph, bit);
           if (lane == 0) {
-            if (j >= 32) ph = __ldcg(wa0 + p.npad + j);
+            if (j0 > 0 || j >= 32) ph = __ldcg(wa0 + p.npad + j);      // (jph: positions 0..31, of the first round)
             sm.misc[13] = ph;
           }
         }

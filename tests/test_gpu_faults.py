@@ -42,3 +42,34 @@ def test_pages_of_the_score_pass_are_read_before_they_are_replaced():
         first = out.clone() if first is None else first
         assert torch.equal(out, first), step
     assert plan.last_status() == 0
+
+
+def test_pivot_behind_walk_entries_that_are_all_members():
+    # 60 of 100 middle tokens are top-k and the base walk begins with 24 to 31 of them: its first residual token lies
+    # behind the entries that were laid out ahead (24 here), but below position 32.  The residual rows are all alike, so
+    # around the right pivot (one of them) both variances are exactly zero, and so are the budgets; around a top-k row
+    # they are rounding errors of its weight.
+    from oracle import vattn_oracle as O
+    from helpers import run_gpu
+    from paper_2510_05688_b200 import synth
+    H, d, n, sink, window, k = 8, 64, 112, 4, 8, 60
+    case = synth.make_case("pivot", dtype="bf16", B=1, Hq=H, Hkv=H, d=d, seq_lens=[n], sink=sink, window=window, k=k,
+                           eps=0.05, delta=0.05, seed=77, gen_seed=1, params=dict(base_rate=0.08))
+    q = case.values(case.q)
+    K, V = np.zeros((H, n, d), np.float32), np.ones((H, n, d), np.float32)
+    for h in range(H):
+        order = sink + O.walk_order(n - sink - window, O.walk_round_keys(case.seed, 0, h, 0, 0, 0))
+        first = 24 + h                                     # the walk position of the first residual token
+        members = np.concatenate([order[:first], order[first + 100 - k:]])
+        assert len(members) == k
+        K[h, members] = (3.1 + 0.37 * h) * np.sqrt(d) * q[0, h] / (q[0, h] @ q[0, h])
+        V[h, members] = 1.5 + 0.25 * h
+    pages = n // 16
+    to_pages = lambda x: x.reshape(H, pages, 16, d).transpose(1, 0, 2, 3)
+    case.k_cache, case.v_cache = case.k_cache.copy(), case.v_cache.copy()
+    case.k_cache[case.block_table[0, :pages]] = synth.f32_to_bf16_bits(to_pages(K))
+    case.v_cache[case.block_table[0, :pages]] = synth.f32_to_bf16_bits(to_pages(V))
+    out, dbg, plan = run_gpu(case)
+    assert (dbg["topk_cnt"] == k).all() and (dbg["base_cnt"] == 3).all() and plan.last_status() == 0
+    assert (dbg["stats"][0, :, 1:3] == 0.0).all()
+    assert (dbg["budgets"][0, :, :3] == 0).all()
