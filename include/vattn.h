@@ -131,7 +131,9 @@ void   vattn_plan_destroy(vattn_plan* plan);
 /* Bytes of device scratch a plan needs (a pure function of the shape), and handing it over.
  * The pointer must be 256-byte aligned and stay valid while the plan is used.  The contents need not
  * be initialised: the library clears what it needs on the first call after this one; between calls it expects to
- * find the workspace as it left it. */
+ * find the workspace as it left it (every call, also one that ends early, leaves its counters at zero; a call recorded
+ * into a caller's graph relies on that too).  Plans that take turns on one piece of memory hand it over again with
+ * this call, each before its turn; a graph recorded right after it carries the clearing. */
 size_t vattn_workspace_bytes(const vattn_plan* plan);
 int    vattn_set_workspace(vattn_plan* plan, void* dev_ptr, size_t bytes);
 
@@ -239,8 +241,8 @@ int vattn_probe_bounded_wait(vattn_plan* plan, uint32_t spins, uint32_t* ran_out
 int vattn_last_launch_count(const vattn_plan* plan);
 
 /* Measurement aid: while kernels > 0, vattn_decode enqueues only its first `kernels` kernels (in the order
- * listed for vattn_set_profiling below) and leaves `out` untouched; 0 restores the whole step.  Lets a
- * harness time one kernel launched back to back, without the launch gaps that events inside a step see.
+ * listed for vattn_set_profiling below), clears the step's counters behind them and leaves `out` untouched; 0 restores
+ * the whole step.  Lets a harness time one kernel launched back to back, without the launch gaps that events inside a step see.
  * Errors: INVALID_ARG (kernels outside [0, VATTN_NUM_KERNELS]). */
 int vattn_set_stop_after(vattn_plan* plan, int kernels);
 

@@ -222,21 +222,27 @@ int check_common(const vattn_plan* pl, const void* q, const void* kc, const void
 #define CU(x) do { if ((x) != cudaSuccess) return VATTN_ERR_CUDA; } while (0)
 
 // The status word and the step's counters and words are cleared once after the workspace is bound; from then on every
-// step finds them at zero because the step before left them so.  (`partial`: a step that will not run to its end.)
-int prepare_stream(vattn_plan* pl, const Prob& p, cudaStream_t st, bool partial) {
+// call finds them at zero because the call before left them so.  That holds for every call, also one that was cut
+// short: a graph that a caller recorded earlier carries no clearing of its own.
+int prepare_stream(vattn_plan* pl, const Prob& p, cudaStream_t st) {
   if (!pl->status_ready) {
     CU(cudaMemsetAsync(p.status, 0, sizeof(unsigned), st));
     pl->status_ready = true;
   }
-  if (!pl->clean || partial) {
+  if (!pl->clean) {
     CU(cudaMemsetAsync(p.m_ord, 0, pl->zero_bytes, st));
     // (recorded into a caller's graph, the clearing belongs to that graph: calls outside it do their own)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CU(cudaStreamIsCapturing(st, &cs));
     pl->clean = cs == cudaStreamCaptureStatusNone;
   }
-  if (partial) pl->clean = false;
   return VATTN_OK;
+}
+// a step that does not run to its end (the measurement aid, an error between two launches) clears behind its last kernel
+int cut_short(vattn_plan* pl, const Prob& p, cudaStream_t st, bool was_clean, int rc) {
+  const cudaError_t e = cudaMemsetAsync(p.m_ord, 0, pl->zero_bytes, st);
+  pl->clean = was_clean && e == cudaSuccess;
+  return rc != VATTN_OK || e == cudaSuccess ? rc : VATTN_ERR_CUDA;
 }
 
 }  // namespace
@@ -425,33 +431,26 @@ int vattn_decode(vattn_plan* plan, const void* q, const void* k_cache, const voi
     p.sel_cap = cap < VATTN_SEL_MINCAP ? VATTN_SEL_MINCAP : cap;
   }
   plan->last_launches = 0;
-  rc = prepare_stream(plan, p, st, plan->stop_after != 0);
+  rc = prepare_stream(plan, p, st);
   if (rc != VATTN_OK) return rc;
   const bool was_clean = plan->clean;
-  plan->clean = false;                        // until the last kernel is enqueued
   prof_mark(plan, 0, st);
   // score pass (walk tokens beside it) -> selection and sample lists (one CTA per head) -> deterministic and
   // base-sample rows (started per head by flags of the selection kernel), budget by the last CTA of a head -> final
   // sample, combination.  Every kernel is launched with programmatic dependent launch: its prologue
   // runs while its predecessor drains; the first one waits before it reads or writes anything.
-  CU(launch_score(p, st));            plan->last_launches++;
-  prof_mark(plan, 1, st);
-  if (plan->stop_after == 1) return VATTN_OK;
-  if (p.dbg.scores)
-    CU(cudaMemcpy2DAsync(p.dbg.scores, sizeof(float) * (size_t)p.max_seq_len, p.scores, sizeof(float) * (size_t)p.npad,
-                         sizeof(float) * (size_t)p.max_seq_len, (size_t)p.B * p.Hq, cudaMemcpyDeviceToDevice, st));
-  CU(launch_walk(p, st));             plan->last_launches++;
-  prof_mark(plan, 2, st);
-  if (plan->stop_after == 2) return VATTN_OK;
-  CU(launch_select(p, st));           plan->last_launches++;
-  prof_mark(plan, 3, st);
-  if (plan->stop_after == 3) return VATTN_OK;
-  CU(launch_stats(p, st));            plan->last_launches++;
-  prof_mark(plan, 4, st);
-  if (plan->stop_after == 4) return VATTN_OK;
-  CU(launch_gather(p, st));           plan->last_launches++;
-  plan->clean = was_clean;
-  prof_mark(plan, 5, st);
+  cudaError_t (*const launch[VATTN_NUM_KERNELS])(const Prob&, cudaStream_t) = {launch_score, launch_walk, launch_select,
+                                                                              launch_stats, launch_gather};
+  for (int i = 0; i < VATTN_NUM_KERNELS; ++i) {
+    if (launch[i](p, st) != cudaSuccess) return cut_short(plan, p, st, was_clean, VATTN_ERR_CUDA);
+    plan->last_launches++;
+    prof_mark(plan, i + 1, st);
+    if (plan->stop_after == i + 1 && i + 1 < VATTN_NUM_KERNELS) return cut_short(plan, p, st, was_clean, VATTN_OK);
+    if (i == 0 && p.dbg.scores &&
+        cudaMemcpy2DAsync(p.dbg.scores, sizeof(float) * (size_t)p.max_seq_len, p.scores, sizeof(float) * (size_t)p.npad,
+                          sizeof(float) * (size_t)p.max_seq_len, (size_t)p.B * p.Hq, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+      return cut_short(plan, p, st, was_clean, VATTN_ERR_CUDA);
+  }
   if (plan->profiling && plan->prof_calls < kProfCalls) plan->prof_calls++;
   return VATTN_OK;
 }
@@ -464,7 +463,7 @@ int vattn_dense_decode(vattn_plan* plan, const void* q, const void* k_cache, con
   Prob p;
   fill_prob(plan, p, q, k_cache, v_cache, block_table, seq_lens, out);
   plan->last_launches = 0;
-  rc = prepare_stream(plan, p, st, false);
+  rc = prepare_stream(plan, p, st);
   if (rc != VATTN_OK) return rc;
   int launches = 0;
   CU(launch_dense(p, st, &launches));

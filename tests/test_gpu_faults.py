@@ -73,3 +73,46 @@ def test_pivot_behind_walk_entries_that_are_all_members():
     assert (dbg["topk_cnt"] == k).all() and (dbg["base_cnt"] == 3).all() and plan.last_status() == 0
     assert (dbg["stats"][0, :, 1:3] == 0.0).all()
     assert (dbg["budgets"][0, :, :3] == 0).all()
+
+
+@pytest.mark.parametrize("stop", [1, 2, 3, 4])
+def test_recorded_step_after_a_step_that_was_cut_short(stop):
+    # a caller's graph carries no clearing of the step's counters: the measurement aid, called between two replays with
+    # another query, left a used-up unit counter and the maxima of its own scores to the next replay
+    import torch
+    from paper_2510_05688_b200 import binding as vb
+    from paper_2510_05688_b200 import synth
+    case = synth.make_case("cut", dtype="bf16", B=6, Hq=8, Hkv=2, d=128, seq_lens=[9000, 20000, 700, 30000, 1, 8191], sink=4,
+                           window=8, k=100, eps=0.05, delta=0.05, seed=5, gen_seed=6,
+                           heavy=dict(R=12, c1=5.0, alpha=(0.75, 1.25)), params=dict(base_rate=0.05))
+    dev = vb.case_to_device(case)
+    plan = vb.plan_for_case(case)
+    plan.set_params(**case.params)
+    q1, q2 = dev["q"], 60.0 * dev["q"].flip(1)       # (far larger scores)
+    q, out = q1.clone(), torch.empty_like(q1)
+    stream = torch.cuda.Stream()
+
+    def step():
+        plan.decode(q, dev["k_cache"], dev["v_cache"], dev["block_table"], dev["seq_lens"], case.sink, case.window, case.k,
+                    case.eps, case.delta, case.seed, out, stream=stream)
+
+    step()
+    torch.cuda.synchronize()
+    want = out.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        step()
+    for _ in range(2):
+        q.copy_(q2)
+        torch.cuda.synchronize()
+        plan.set_stop_after(stop)
+        step()
+        plan.set_stop_after(0)
+        torch.cuda.synchronize()
+        q.copy_(q1)
+        out.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+    assert plan.last_status() == 0
