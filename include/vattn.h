@@ -132,8 +132,9 @@ void   vattn_plan_destroy(vattn_plan* plan);
  * The pointer must be 256-byte aligned and stay valid while the plan is used.  The contents need not
  * be initialised: the library clears what it needs on the first call after this one; between calls it expects to
  * find the workspace as it left it (every call, also one that ends early, leaves its counters at zero; a call recorded
- * into a caller's graph relies on that too).  Plans that take turns on one piece of memory hand it over again with
- * this call, each before its turn; a graph recorded right after it carries the clearing. */
+ * into a caller's graph relies on that too).  Plans may take turns on one piece of memory: while the workspaces of two
+ * live plans overlap, every call of theirs clears first (record a caller's graph after the last of them was handed the
+ * memory; the status bits of such plans are not kept). */
 size_t vattn_workspace_bytes(const vattn_plan* plan);
 int    vattn_set_workspace(vattn_plan* plan, void* dev_ptr, size_t bytes);
 

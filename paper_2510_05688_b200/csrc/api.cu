@@ -2,6 +2,7 @@
 // decode step.  Host code only; no device memory is allocated or freed here.
 #include <math.h>
 #include <new>
+#include <pthread.h>
 #include <string.h>
 #include "vattn_internal.cuh"
 
@@ -13,6 +14,8 @@ struct vattn_plan {
   size_t ws_bytes;
   bool status_ready;
   bool clean;             // the step's counters and words are known to be zero (every step leaves them so)
+  int shared;             // another plan's workspace overlaps this one's: every call clears first (see bind_workspace)
+  vattn_plan* next;       // list of the plans that have a workspace
   int last_launches;
   double z_delta_of, z[17];  // normal quantiles for the last delta
   // optional per-kernel timing (events are created on first use; no device memory involved)
@@ -221,20 +224,48 @@ int check_common(const vattn_plan* pl, const void* q, const void* kc, const void
 
 #define CU(x) do { if ((x) != cudaSuccess) return VATTN_ERR_CUDA; } while (0)
 
+// The plans that have a workspace.  `shared` of a plan: 0 no other live plan's workspace overlaps its own, 1 one does,
+// 2 one did (its counters are cleared once more).
+pthread_mutex_t g_bound_lock = PTHREAD_MUTEX_INITIALIZER;
+vattn_plan* g_bound = nullptr;
+inline int shared_state(const vattn_plan* pl) { return __atomic_load_n(&pl->shared, __ATOMIC_ACQUIRE); }
+inline bool overlap(const vattn_plan* a, const void* ws, size_t bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a->ws), y = reinterpret_cast<uintptr_t>(ws);
+  return x < y + bytes && y < x + a->total;
+}
+void bind_workspace(vattn_plan* pl, void* ws, size_t bytes) {       // (ws null: the plan gives its workspace up)
+  pthread_mutex_lock(&g_bound_lock);
+  for (vattn_plan** at = &g_bound; *at; at = &(*at)->next)
+    if (*at == pl) { *at = pl->next; break; }
+  const void* old = pl->ws;
+  pl->ws = ws; pl->ws_bytes = bytes;
+  if (ws) { pl->next = g_bound; g_bound = pl; }
+  for (vattn_plan* a = g_bound; a; a = a->next) {
+    if (a != pl && !overlap(a, ws, pl->total) && !(old && overlap(a, old, pl->total))) continue;
+    int now = shared_state(a) != 0 ? 2 : 0;
+    for (const vattn_plan* o = g_bound; o; o = o->next) if (o != a && overlap(a, o->ws, o->total)) { now = 1; break; }
+    __atomic_store_n(&a->shared, now, __ATOMIC_RELEASE);
+  }
+  pthread_mutex_unlock(&g_bound_lock);
+}
+
 // The status word and the step's counters and words are cleared once after the workspace is bound; from then on every
 // call finds them at zero because the call before left them so.  That holds for every call, also one that was cut
-// short: a graph that a caller recorded earlier carries no clearing of its own.
+// short: a graph that a caller recorded earlier carries no clearing of its own.  Plans that take turns on one piece of
+// memory write over each other's counters, so each of their calls clears first.
 int prepare_stream(vattn_plan* pl, const Prob& p, cudaStream_t st) {
   if (!pl->status_ready) {
     CU(cudaMemsetAsync(p.status, 0, sizeof(unsigned), st));
     pl->status_ready = true;
   }
-  if (!pl->clean) {
+  int sh = shared_state(pl);
+  if (!pl->clean || sh != 0) {
     CU(cudaMemsetAsync(p.m_ord, 0, pl->zero_bytes, st));
     // (recorded into a caller's graph, the clearing belongs to that graph: calls outside it do their own)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CU(cudaStreamIsCapturing(st, &cs));
     pl->clean = cs == cudaStreamCaptureStatusNone;
+    if (sh == 2 && pl->clean) __atomic_compare_exchange_n(&pl->shared, &sh, 0, false, __ATOMIC_ACQ_REL, __ATOMIC_ACQUIRE);
   }
   return VATTN_OK;
 }
@@ -305,6 +336,7 @@ int vattn_plan_create(const vattn_shape* shape, vattn_plan** out) {
 
 void vattn_plan_destroy(vattn_plan* plan) {
   if (!plan) return;
+  if (plan->ws) bind_workspace(plan, nullptr, 0);
   for (auto& e : plan->host_steps)
     if (e.used && e.exec) cudaGraphExecDestroy(e.exec);
   if (plan->ev) {
@@ -356,8 +388,7 @@ size_t vattn_workspace_bytes(const vattn_plan* plan) { return plan ? plan->total
 int vattn_set_workspace(vattn_plan* plan, void* dev_ptr, size_t bytes) {
   if (!plan) return VATTN_ERR_INVALID_ARG;
   if (!dev_ptr || misaligned(dev_ptr, 256) || bytes < plan->total) return VATTN_ERR_WORKSPACE;
-  plan->ws = dev_ptr;
-  plan->ws_bytes = bytes;
+  bind_workspace(plan, dev_ptr, bytes);
   plan->status_ready = false;
   plan->clean = false;
   plan->gen++;
@@ -549,7 +580,8 @@ int vattn_decode_host(vattn_plan* plan, const void* q_host, const void* k_cache,
   // page-locked host buffers, outside any capture of the caller, and with no introspection switched on.
   vattn_plan::HostStep* e = nullptr;
   const vattn_debug& dg = plan->dbg;
-  const bool plain_only = plan->profiling || plan->stop_after != 0 || dg.kernel_ticks || dg.topk_idx || dg.topk_cnt ||
+  // (nor with a workspace that other plans write to: a recorded step may carry no clearing)
+  const bool plain_only = shared_state(plan) != 0 || plan->profiling || plan->stop_after != 0 || dg.kernel_ticks || dg.topk_idx || dg.topk_cnt ||
                           dg.base_idx || dg.base_cnt || dg.dyn_idx || dg.dyn_cnt || dg.budgets || dg.stats || dg.scores ||
                           dg.paths;
   if (!plain_only) {

@@ -171,7 +171,8 @@ __global__ void __launch_bounds__(SCORE_THREADS, 2) k_score_stream(const __grid_
         }
       }
       ++ucount;
-      u = (int)gridDim.x + (int)__shfl_sync(0xFFFFFFFFu, nxt, 0);
+      nxt = __shfl_sync(0xFFFFFFFFu, nxt, 0);
+      u = nxt >= (unsigned)U ? U : (int)(gridDim.x + nxt);       // (a counter that somebody wrote over ends the loop)
     }
     if (first) pdl_trigger();
     // one end mark per consumer (consumer w owns the stages i = w mod CWN)

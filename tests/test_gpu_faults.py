@@ -116,3 +116,50 @@ def test_recorded_step_after_a_step_that_was_cut_short(stop):
         torch.cuda.synchronize()
         assert torch.equal(out, want)
     assert plan.last_status() == 0
+
+
+def test_plans_that_take_turns_on_one_workspace():
+    # two plans of other shapes on the same memory: each finds the other's scores and lists where its own counters are
+    # (unit counters and maxima that are not zero), whichever ran last, through both entry points, and when one is gone
+    import torch
+    from helpers import out_values, run_oracle
+    from paper_2510_05688_b200 import binding as vb
+    from paper_2510_05688_b200 import synth
+    kw = dict(d=64, sink=4, window=8, k=16, eps=0.05, delta=0.05, seed=1, params=dict(base_rate=0.05))
+    cases = [synth.make_case("a", dtype="bf16", B=3, Hq=8, Hkv=2, seq_lens=[5000, 333, 0], gen_seed=1, **kw),
+             synth.make_case("b", dtype="bf16", B=2, Hq=4, Hkv=4, seq_lens=[900, 2500], gen_seed=2, **kw)]
+    want = [out_values(c, run_oracle(c)[0]) for c in cases]
+    devs = [vb.case_to_device(c) for c in cases]
+    plans = [vb.Plan(batch=c.batch, num_q_heads=c.num_q_heads, num_kv_heads=c.num_kv_heads, head_dim=64,
+                     max_blocks_per_seq=c.max_blocks_per_seq, num_blocks=c.num_blocks, max_seq_len=c.max_blocks_per_seq * 16,
+                     dtype=vb.DTYPE_BF16, alloc_workspace=False) for c in cases]
+    need = max(p.workspace_bytes() for p in plans)
+    mem = torch.empty(need + 4096, dtype=torch.uint8, device="cuda")
+    plans[0].set_workspace(mem.data_ptr(), need)
+    plans[1].set_workspace(mem.data_ptr() + 4096, need)              # (overlapping, not the same address)
+    pinned = [{x: dv[x].cpu().pin_memory() for x in ("q", "block_table", "seq_lens")} for dv in devs]
+    stream = torch.cuda.Stream()
+
+    def run(i, host):
+        c, dv, p = cases[i], devs[i], plans[i]
+        p.set_params(**c.params)
+        scalars = (c.sink, c.window, c.k, c.eps, c.delta, c.seed)
+        torch.cuda.synchronize()
+        if host:
+            out = torch.empty_like(pinned[i]["q"]).pin_memory()
+            for _ in range(3):
+                p.decode_host(pinned[i]["q"], dv["k_cache"], dv["v_cache"], pinned[i]["block_table"], pinned[i]["seq_lens"],
+                              *scalars, out, stream=stream)
+        else:
+            out = torch.empty_like(dv["q"])
+            p.decode(dv["q"], dv["k_cache"], dv["v_cache"], dv["block_table"], dv["seq_lens"], *scalars, out)
+        torch.cuda.synchronize()
+        got = out_values(c, out.view(torch.int16).cpu().numpy().view(np.uint16))
+        assert np.abs(got - want[i]).max() <= 2e-2, (i, host)
+
+    for host in (False, True, False):
+        for i in (0, 1, 0, 0, 1, 1):
+            run(i, host)
+    del plans[1]                                                     # (its counters are still lying there)
+    run(0, False)
+    run(0, True)
