@@ -392,12 +392,14 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
   }
   const float m_f = unord_f32(__ldcg(p.m_ord + bh));
   __syncthreads();
-  if (s_word == 0ull) {                            // the bounded wait ran out
+  unsigned long long word = s_word;
+  if (word == 0ull) {                              // the bounded wait ran out
     pdl_wait();
+    __syncthreads();                               // (every thread has seen the zero before it is replaced)
     if (tid == 0) s_word = base_cta ? __ldcg(&hw->sample) : (unsigned long long)__ldcg(&hw->topk);
     __syncthreads();
+    word = s_word;
   }
-  const unsigned long long word = s_word;
   if (base_cta) DBGT(36);
   if (base_cta && split == 0) DBGH(bh, 6);
   const bool odd = ((word >> (base_cta ? 2 : 1)) & 1ull) != 0;       // the KV head's K holds elements that are not finite

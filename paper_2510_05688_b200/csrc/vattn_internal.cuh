@@ -514,7 +514,10 @@ __device__ __forceinline__ unsigned long long wait_word64(const unsigned long lo
   asm volatile("fence.acq_rel.gpu;" ::: "memory");
   return v;
 }
-constexpr unsigned VATTN_WORD_SPINS = 1u << 16;   // polls of a published word (about 10 ms) before the fallback
+#ifndef VATTN_WORD_POLLS
+#define VATTN_WORD_POLLS (1u << 16)    // (a build with -DVATTN_WORD_POLLS=1 takes the fallbacks nearly everywhere: same results)
+#endif
+constexpr unsigned VATTN_WORD_SPINS = VATTN_WORD_POLLS;   // polls of a published word (about 10 ms) before the fallback
 
 // A head's GMeta as one 16-byte word, so that the poll that sees it also has it: 19 bits each of b, n_s and L, list,
 // empty row, "start is not zero", valid; the bits of m; W1.  One thread, behind a barrier (the fence is cumulative).
