@@ -143,3 +143,17 @@ def test_plans_and_partial_steps_in_turn_on_one_stream():
             diff = np.abs(out_values(c, got) - out_values(c, ref))
             assert diff.max() <= (2e-2 if c.dtype == "bf16" else 1e-5 * np.abs(out_values(c, ref)).max()), rep
             assert p.last_status() == 0
+
+
+@pytest.mark.parametrize("dtype,n", [("bf16", 2400), ("bf16", 33000), ("fp32", 5000), ("bf16", 131073)])
+@pytest.mark.parametrize("offset", [5.0, 40.0])
+def test_logits_with_a_common_offset(dtype, n, offset):
+    # queries and keys share a component: every logit is the offset and a little, so the sample's keys crowd into one bin
+    # of the top 12 bits and the bound comes from the next 12
+    case = small(dtype, [n], Hq=2, Hkv=1, d=64, k=n // 40, key_std=0.1, heavy=None, params=dict(base_rate=0.02))
+    a = np.sqrt(offset * 8.0 / 64.0)
+    store = synth.f32_to_bf16_bits if dtype == "bf16" else (lambda x: x.astype(np.float32))
+    case.q, case.k_cache = store(case.values(case.q) + np.float32(a)), store(case.values(case.k_cache) + np.float32(a))
+    _, dbg, det, plan = check(case)
+    assert det[(0, 0)]["m"] > 0.6 * offset and plan.last_status() == 0
+    assert (dbg["paths"] & 17 != 0).all()
