@@ -229,19 +229,26 @@ __device__ __noinline__ Found select_general(const Prob& p, unsigned char* smem,
   float hi, lo;
   int nbt, band_mode = 0;
   const int PT = (mlen + NT - 1) / NT;               // keys per thread
-  // every key of the middle range, in token order per thread: f(u, token, valid, key); uniform trip count
+  // every key of the middle range, in token order per thread: f(u, token, valid, key); uniform trip count, four scores
+  // requested at a time
   auto for_slice = [&](auto f) {
 #pragma unroll 1
-    for (int u = 0; u < PT; ++u) {
-      const int i = s0 + tid + NT * u;
-      const bool v = i < l_start;
-      // (a NaN score ranks below everything: the lists stay complete whatever the inputs hold)
-      const float s = v ? __ldg(sc + i) : 0.f;
-      f(u, i, v, v ? ~ord_f32(s == s ? s : -CUDART_INF_F) : 0xFFFFFFFFu);
+    for (int u0 = 0; u0 < PT; u0 += 4) {
+      float s[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) { const int i = s0 + tid + NT * (u0 + e); s[e] = i < l_start ? __ldg(sc + i) : 0.f; }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int u = u0 + e, i = s0 + tid + NT * u;
+        if (u >= PT) break;
+        const bool v = i < l_start;
+        // (a NaN score ranks below everything: the lists stay complete whatever the inputs hold)
+        f(u, i, v, v ? ~ord_f32(s[e] == s[e] ? s[e] : -CUDART_INF_F) : 0xFFFFFFFFu);
+      }
     }
   };
-  const float gamma = sm.gamma[0] >= 0.f ? sm.gamma[0] : 0.f;      // (NaN: non-finite inputs)
   __syncthreads();
+  const float gamma = sm.gamma[0] >= 0.f ? sm.gamma[0] : 0.f;      // (NaN: non-finite inputs)
   int* cntM = p.sel_cnt + (long long)bh * 2 * (p.npad / 16 + 32);                                 // [PT * NWARP] tokens above the band per (u, warp), then its scan
   int* cntB = cntM + p.npad / 16 + 32;                         // the same for the band
   if (kk == mlen) { hi = -CUDART_INF_F; lo = -CUDART_INF_F; }
@@ -449,8 +456,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
   int path = 0;
   float hi = CUDART_INF_F, lo = CUDART_INF_F;          // members: s > hi; near-tie band: lo <= s <= hi
   int nbt = 0, band_mode = 0;
-  const bool usual = kk > 0 && kk < mlen;              // there is a threshold to find
-  bool general = kk > 0 && kk == mlen;
+  // There is a threshold to find, and the list is likely to hold what the bound lets through (see sel_cap in api.cu).  A
+  // top-k set of a tenth of 131,071 tokens mostly overflows it: 622 us per step of 32 heads when that was found out only
+  // after the compare pass, 600 like this, and 522 with the general case's scores requested four at a time.
+  const int stride = sample_stride(n, SAMPLES);
+  const float through = (float)kk + 4.f * __fsqrt_rn((float)kk * (float)stride) + 9.f * (float)stride;
+  const bool usual = kk > 0 && kk < mlen && (mlen <= cap || through + 2.f * __fsqrt_rn(through * (float)stride) <= (float)cap);
+  bool general = kk > 0 && !usual;
   if (!usual && warp == NWARP - 1 && lane == 0)
     sm.gamma[0] = __double2float_ru(gfac * (double)__uint_as_float(kmax_bits));
 
@@ -472,7 +484,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
     // against one another took 106 instead of 72 us per step at 32 heads x 32,768 tokens with logits around 20, and 780 instead
     // of 176 at 131,071.)
     if (mlen > cap) {
-      const int stride = sample_stride(n, SAMPLES), ns_all = (n + stride - 1) / stride;
+      const int ns_all = (n + stride - 1) / stride;
       unsigned kept[SAMPLES / NT];             // (all ones: not a middle token)
 #pragma unroll
       for (int e = 0; e < SAMPLES / NT; ++e) {

@@ -157,3 +157,12 @@ def test_logits_with_a_common_offset(dtype, n, offset):
     _, dbg, det, plan = check(case)
     assert det[(0, 0)]["m"] > 0.6 * offset and plan.last_status() == 0
     assert (dbg["paths"] & 17 != 0).all()
+
+
+@pytest.mark.parametrize("dtype,n,k", [("bf16", 131073, 20000), ("bf16", 40000, 17000), ("fp32", 33000, 15000), ("bf16", 20000, 12000)])
+def test_top_k_sets_around_the_candidate_list(dtype, n, k):
+    # more members than the list of 16,384 candidates takes (or may take): the general selection with a threshold; 12,000
+    # of 20,000 tokens: the usual one with an almost full list
+    _, dbg, _, plan = check(small(dtype, [n], Hq=2, Hkv=1, d=64, k=k, params=dict(base_rate=0.02)))
+    assert plan.last_status() == 0
+    assert ((dbg["paths"] & 17 != 0) == (n == 20000)).all()
