@@ -166,3 +166,15 @@ def test_top_k_sets_around_the_candidate_list(dtype, n, k):
     _, dbg, _, plan = check(small(dtype, [n], Hq=2, Hkv=1, d=64, k=k, params=dict(base_rate=0.02)))
     assert plan.last_status() == 0
     assert ((dbg["paths"] & 17 != 0) == (n == 20000)).all()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("eps", [0.07, 0.03])
+def test_lists_from_laid_out_walk_entries(dtype, eps):
+    # half of the tokens are top-k: more than 1,024 marked entries in the final sample's array, so every budget is served
+    # from a list, inside the array (8 base budgets) and beyond it
+    case = small(dtype, [12000], Hq=2, Hkv=1, d=64, k=6000, key_std=0.1, heavy=None, eps=eps, delta=eps)
+    _, dbg, det, plan = check(case)
+    for r in det.values():
+        assert r["b0"] < r["b"] < 8 * r["b0"] if eps == 0.07 else 8 * r["b0"] < r["b"] < r["n_s"]
+    assert plan.last_status() == 0
