@@ -91,15 +91,18 @@ void derive(vattn_plan* pl) {
   pl->dense_splits = sp < 1 ? 1 : (sp > 128 ? 128 : sp);
   // statistics kernel (128-thread CTAs, 5 per SM): one wave for both kinds of CTA, half each, on the SMs that the selection
   // leaves free (with few heads it holds one SM per head until after the rows have been published: CTAs beyond that
-  // started 4 us late; 151.9 -> 148.5 us per step at 32 heads of 131,071 tokens, others within 1 %).  When four
-  // CTAs per kind and head overfill the wave the kernel is throughput-bound: four all the same, so that the first heads'
-  // budgets come early (2: 116 instead of 110 us at 128 heads x 32,768, 6: 112), but two from 186 heads and one from
-  // 371 on, where the waits, partials and tickets of twice the CTAs cost more (208.9 -> 205.3 us at 256 x 32,768,
-  // 628 -> 617 at 1,024 x 4,096 to 32,768; one at 256 x 32,768: 212).
+  // started 4 us late; 151.9 -> 148.5 us per step at 32 heads of 131,071 tokens, others within 1 %).  From 70 heads on
+  // four CTAs per kind and head overfill that wave and the kernel is throughput-bound: four all the same, so that the first
+  // heads' budgets come early (2: 116 instead of 110 us at 128 heads x 32,768, 6: 112), but two where four would be two
+  // waves of all SMs (186 heads) and one where two would be (371), where the waits, partials and tickets of twice the CTAs
+  // cost more (4 -> 2: 208.9 -> 205.3 us at 256 x 32,768, one there: 212; 2 -> 1: 628 -> 617 at 1,024 x 4,096 to 32,768).
+  // Both lines at three quarters of these counts: 79.9 instead of 75.2 us at 288 x 2,049 and 220 instead of 210 at 288 x
+  // 4,096 to 32,768, 154.4 instead of 151.7 at 144 x 32,768; 175.5 instead of 177.3 at 184.
   {
     const int sms = device_sm_count(), wave = 5 * (sms - (heads < sms / 4 ? heads : sms / 4)) / heads;
     if (wave < 8) {
-      pl->stat_splits = pl->stat_splits_base = wave < 2 ? 1 : wave < 4 ? 2 : 4;
+      const int full = 5 * sms / heads;
+      pl->stat_splits = pl->stat_splits_base = full < 2 ? 1 : full < 4 ? 2 : 4;
     } else {
       const int sb = (wave + 1) / 2;
       pl->stat_splits_base = sb > VATTN_STAT_MAXS ? VATTN_STAT_MAXS : sb;
@@ -426,7 +429,8 @@ int vattn_decode(vattn_plan* plan, const void* q, const void* k_cache, const voi
   fill_prob(plan, p, q, k_cache, v_cache, block_table, seq_lens, out);
   p.sink = sink; p.window = window; p.k = k;
   {
-    // statistics kernel: never more CTAs than rows warrant (about 64 deterministic, 48 base-sample rows each)
+    // statistics kernel: never more CTAs than the longest sequence's rows warrant, 64 deterministic or 48 base-sample rows
+    // each (a head uses fewer where its own rows are fewer than stat_rows each)
     const double msl = (double)plan->shape.max_seq_len;
     double kmax = plan->params.topk_frac > 0.f ? floor((double)plan->params.topk_frac * msl) : (double)k;
     double rows = (double)sink + (double)window + kmax;

@@ -27,7 +27,7 @@ def test_candidate_bound_sizes(n, heads, kv):
 
 @pytest.mark.parametrize("B,Hq", [(37, 4), (149, 1), (37, 8), (297, 1), (160, 8)])
 def test_head_counts_of_the_selection_and_the_walk(B, Hq):
-    # 148 | 149 | 296 | 297 heads: other block sizes of the selection; 1,280 heads share 1,184 walk CTAs
+    # 296 | 297 heads: other block sizes of the selection on plans for short sequences; 1,280 heads share 1,184 walk CTAs
     lens = [(37 * i) % 700 + 1 for i in range(B)]
     check(small("bf16", lens, Hq=Hq, Hkv=1, d=64, k=9))
 
@@ -51,8 +51,8 @@ def test_many_heads_with_shares_of_whole_sections():
 @pytest.mark.parametrize("B,Hq", [(4, 4), (17, 1), (8, 4), (11, 3), (32, 4), (43, 3), (40, 4), (23, 7),
                                   (37, 5), (62, 3), (74, 5), (53, 7), (64, 8)])
 def test_head_counts_of_the_gather_and_the_statistics(B, Hq):
-    # 16 | 17, 32 | 33 heads: other chunk counts and the other decomposition of the gather; 128 | 129: rows per statistics
-    # CTA, 185 | 186 and 370 | 371: its CTAs per head; 160 | 161 and 512: the gather's least chunk (128, 256, 512 rows)
+    # 16 | 17, 32 | 33 heads: other chunk counts and the other decomposition of the gather; 160 | 161 and 512: its least
+    # chunk (128, 256, 512 rows); 128 | 129: rows per statistics CTA
     lens = [(53 * i) % 500 + 300 for i in range(B - 1)] + [1200]
     case = small("bf16", lens, Hq=Hq, Hkv=1, d=64, k=9)
     for budget in (129, 257, 513):
@@ -178,3 +178,20 @@ def test_lists_from_laid_out_walk_entries(dtype, eps):
     for r in det.values():
         assert r["b0"] < r["b"] < 8 * r["b0"] if eps == 0.07 else 8 * r["b0"] < r["b"] < r["n_s"]
     assert plan.last_status() == 0
+
+
+@pytest.mark.parametrize("B,Hq", [(8, 16), (37, 5), (62, 3), (37, 10), (53, 7)])
+def test_statistics_ctas_per_head(B, Hq):
+    # 128 and 185 heads: four CTAs per kind and head; 186, 370: two; 371: one; with rows for more than four of either kind
+    # (256 rows each, 64 up to 128 heads)
+    case = small("bf16", [4000 - 3 * i for i in range(B)], Hq=Hq, Hkv=1, d=64, k=1300, params=dict(base_rate=0.45))
+    _, dbg, _, _ = check(case)
+    assert (dbg["topk_cnt"] > 4 * 256).all() and (dbg["base_cnt"] > 4 * 256).all()
+
+
+@pytest.mark.parametrize("B,Hq,tokens", [(37, 2, 16400), (15, 5, 16400), (15, 5, 65536), (15, 5, 65552), (37, 4, 65552), (149, 1, 65552)])
+def test_block_sizes_of_the_selection(B, Hq, tokens):
+    # 1,024 threads above 16,384 tokens up to 74 heads, above 65,536 up to 148; 512 otherwise (the plan's longest sequence
+    # decides, whatever the sequences are now)
+    lens = [(389 * i) % 3000 + 1 for i in range(B)]
+    check(small("bf16", lens, Hq=Hq, Hkv=1, d=64, k=60, max_blocks=tokens // 16))
