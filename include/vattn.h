@@ -123,8 +123,7 @@ typedef struct {
 /* Create / destroy a plan for one problem shape.  `out` receives a host object.  Errors: INVALID_ARG,
  * UNSUPPORTED (head_dim other than 64 / 128, block_size other than 16, more than 64 (query token, query head)
  * pairs per KV head, q_len above 64, max_seq_len above 262,144, a bf16 batch above 1,536 rows, a batch above
- * 32,767 rows or more than 65,535 (batch row, query token, query head) triples: the kernels' grid dimensions; a cache of
- * more than 2^32 pieces of gcd(page stride, token stride) bytes, which takes 64 GB or more). */
+ * 32,767 rows or more than 65,535 (batch row, query token, query head) triples: the kernels' grid dimensions). */
 int    vattn_plan_create(const vattn_shape* shape, vattn_plan** out);
 void   vattn_plan_destroy(vattn_plan* plan);
 

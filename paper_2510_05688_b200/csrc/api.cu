@@ -144,17 +144,17 @@ void derive(vattn_plan* pl) {
   pl->total = off;
 }
 
-// One 32-bit index per cache row (see Prob::row_unit).  False: the cache has more row_unit-sized pieces than 2^32, which
-// takes more than 64 GB of K per layer with page and token strides that share no factor above 16 bytes.
-bool row_geometry(const vattn_shape& s, long long sb, long long st, unsigned* unit, unsigned* pg, unsigned* tk) {
-  const long long es = s.dtype == VATTN_DTYPE_BF16 ? 2 : 4;
-  long long x = sb * es, y = st * es;
+// One 32-bit index per cache row (see Prob::row_unit)
+void row_geometry(Prob& p, long long es) {
+  p.page_bytes = p.sb * es; p.token_bytes = p.st * es;
+  long long x = p.page_bytes, y = p.token_bytes;
   while (y) { const long long r = x % y; x = y; y = r; }
   while (x > (1ll << 30) && x % 2 == 0) x /= 2;
-  if (x > (1ll << 30)) return false;
-  *unit = (unsigned)x; *pg = (unsigned)(sb * es / x); *tk = (unsigned)(st * es / x);
-  return sb * es / x <= 0xFFFFFFFFll && st * es / x <= 0xFFFFFFFFll &&
-         (double)(s.num_blocks - 1) * (double)(sb * es / x) + 15.0 * (double)(st * es / x) < 4294967296.0;
+  p.row_unit = 0u; p.row_pg = VATTN_BLOCK; p.row_tk = 1u;
+  if (x <= 0 || x > (1ll << 30)) return;
+  const long long pg = p.page_bytes / x, tk = p.token_bytes / x;
+  if (pg < 1 || pg >= 1ll << 32 || tk >= 1ll << 28 || (long long)(p.num_blocks - 1) > ((1ll << 32) - 1 - (VATTN_BLOCK - 1) * tk) / pg) return;
+  p.row_unit = (unsigned)x; p.row_pg = (unsigned)pg; p.row_tk = (unsigned)tk;
 }
 
 int fill_prob(const vattn_plan* pl, Prob& p, const void* q, const void* kc, const void* vc, const int32_t* bt,
@@ -171,7 +171,7 @@ int fill_prob(const vattn_plan* pl, Prob& p, const void* q, const void* kc, cons
   } else {
     p.sb = s.kv_stride_block; p.sh = s.kv_stride_head; p.st = s.kv_stride_token;
   }
-  row_geometry(s, p.sb, p.st, &p.row_unit, &p.row_pg, &p.row_tk);
+  row_geometry(p, s.dtype == VATTN_DTYPE_BF16 ? 2 : 4);
   p.q = q; p.kc = kc; p.vc = vc; p.bt = bt; p.seq_lens = sl; p.out = out;
   p.topk_frac = pr.topk_frac;
   p.base_rate = pr.base_rate > 0.f ? pr.base_rate : 0.025f;
@@ -320,12 +320,6 @@ int vattn_plan_create(const vattn_shape* shape, vattn_plan** out) {
     const int epl = s.dtype == VATTN_DTYPE_BF16 ? 8 : 4;
     if (s.kv_stride_block <= 0 || s.kv_stride_head <= 0 || s.kv_stride_token < s.head_dim) return VATTN_ERR_INVALID_ARG;
     if (s.kv_stride_block % epl || s.kv_stride_head % epl || s.kv_stride_token % epl) return VATTN_ERR_INVALID_ARG;
-  }
-  {
-    const long long st = custom ? s.kv_stride_token : s.head_dim;
-    const long long sb = custom ? s.kv_stride_block : (long long)s.num_kv_heads * s.block_size * s.head_dim;
-    unsigned u, pgm, tkm;
-    if (!row_geometry(s, sb, st, &u, &pgm, &tkm)) return VATTN_ERR_UNSUPPORTED;
   }
   vattn_plan* pl = new (std::nothrow) vattn_plan();
   if (!pl) return VATTN_ERR_INVALID_ARG;

@@ -43,7 +43,7 @@ constexpr int FLAT_MAX_HEADS = VATTN_GATHER_FLAT_HEADS;
 __host__ __device__ constexpr int min_chunk(int heads) { return heads >= 512 ? 512 : heads > 160 ? 256 : 128; }   // per-head decomposition
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-template <typename T, int D, bool KV>
+template <typename T, int D, bool KV, bool SPLIT>
 struct Gather {
   static constexpr int EPL = Elem<T>::EPL, LPR = D / EPL, RPI = 32 / LPR, NE = D + 1;
   static constexpr int WB = RPI * UN, CB = NWARP * WB;      // rows per warp and per CTA of a batch
@@ -149,10 +149,10 @@ struct Gather {
         if (k < nbat) {
           const int4 id = *reinterpret_cast<const int4*>(sm.idx + k * CB + mine);
           uint4 (&dst)[UN][32] = sm.ring[warp][slot_];
-          cp_async16(&dst[0][lane], row_at(p, vb, id.x));
-          cp_async16(&dst[1][lane], row_at(p, vb, id.y));
-          cp_async16(&dst[2][lane], row_at(p, vb, id.z));
-          cp_async16(&dst[3][lane], row_at(p, vb, id.w));
+          cp_async16(&dst[0][lane], row_at<SPLIT>(p, vb, id.x));
+          cp_async16(&dst[1][lane], row_at<SPLIT>(p, vb, id.y));
+          cp_async16(&dst[2][lane], row_at<SPLIT>(p, vb, id.z));
+          cp_async16(&dst[3][lane], row_at<SPLIT>(p, vb, id.w));
         }
         cp_async_commit();
       };
@@ -281,10 +281,10 @@ struct Gather {
     uint4 r[UN];
     auto load = [&](int k) {
       const int4 id = *reinterpret_cast<const int4*>(sm.idx + k * CB + mine);
-      r[0] = __ldcs(reinterpret_cast<const uint4*>(row_at(p, kb, id.x)));
-      r[1] = __ldcs(reinterpret_cast<const uint4*>(row_at(p, kb, id.y)));
-      r[2] = __ldcs(reinterpret_cast<const uint4*>(row_at(p, kb, id.z)));
-      r[3] = __ldcs(reinterpret_cast<const uint4*>(row_at(p, kb, id.w)));
+      r[0] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.x)));
+      r[1] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.y)));
+      r[2] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.z)));
+      r[3] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.w)));
     };
     load(0);
 #pragma unroll 1
@@ -312,9 +312,9 @@ struct Gather {
   }
 };
 
-template <typename T, int D, bool KV>
+template <typename T, int D, bool KV, bool SPLIT>
 __global__ void __launch_bounds__(NT, VATTN_GATHER_CTAS) k_gather(const __grid_constant__ Prob p) {
-  using G = Gather<T, D, KV>;
+  using G = Gather<T, D, KV, SPLIT>;
   __shared__ __align__(16) typename G::Sm sm;
   pdl_trigger();                                        // (the next step's first kernel waits before it touches anything)
   TICK_BEGIN(p, VATTN_K_GATHER);
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(NT, VATTN_GATHER_CTAS) k_gather(const __grid_c
 
 template <typename T, int D, bool KV>
 __global__ void __launch_bounds__(NT, VATTN_GATHER_CTAS) k_gather_flat(const __grid_constant__ Prob p) {
-  using G = Gather<T, D, KV>;
+  using G = Gather<T, D, KV, false>;
   __shared__ __align__(16) typename G::Sm sm;
   pdl_trigger();                                        // (the next step's first kernel waits before it touches anything)
   TICK_BEGIN(p, VATTN_K_GATHER);
@@ -394,24 +394,26 @@ __global__ void __launch_bounds__(NT, VATTN_GATHER_CTAS) k_gather_flat(const __g
 
 }  // namespace
 
+template <typename T, int D, bool KV, bool SPLIT>
+static cudaError_t launch_per_head(const Prob& p, cudaStream_t s) {
+  static size_t have[VATTN_MAXDEV];
+  if (p.gat_slots < MAXS) return cudaErrorInvalidValue;
+  cudaError_t e = optin_smem(k_gather<T, D, KV, SPLIT>, 0, have, true);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_gather<T, D, KV, SPLIT>, dim3(MAXS, p.B * p.Hq), dim3(NT), 0, s, p);
+}
 template <typename T, int D, bool KV>
 static cudaError_t launch_gather_t(const Prob& p, cudaStream_t s) {
   const int BH = p.B * p.Hq;
-  static size_t have[VATTN_MAXDEV], have_flat[VATTN_MAXDEV];
-  if (BH <= FLAT_MAX_HEADS) {
-    // at most gat_slots chunks per head; one wave of CTAs walks them with a grid stride
-    if (p.gat_slots < VATTN_GATHER_FLAT_SLOTS) return cudaErrorInvalidValue;
-    const long long most = (long long)BH * p.gat_slots;
-    cudaError_t e = optin_smem(k_gather_flat<T, D, KV>, 0, have_flat, true);
-    if (e != cudaSuccess) return e;
-    const long long cap = (long long)VATTN_GATHER_CTAS * device_sm_count();
-    const int grid = (int)(most < cap ? most : cap);
-    return launch_pdl(k_gather_flat<T, D, KV>, dim3(grid), dim3(NT), 0, s, p);
-  }
-  if (p.gat_slots < MAXS) return cudaErrorInvalidValue;
-  cudaError_t e = optin_smem(k_gather<T, D, KV>, 0, have, true);
+  if (p.row_unit == 0u) return launch_per_head<T, D, KV, true>(p, s);      // (rare: no flat variant)
+  if (BH > FLAT_MAX_HEADS) return launch_per_head<T, D, KV, false>(p, s);
+  // at most gat_slots chunks per head; one wave of CTAs walks them with a grid stride
+  static size_t have[VATTN_MAXDEV];
+  if (p.gat_slots < VATTN_GATHER_FLAT_SLOTS) return cudaErrorInvalidValue;
+  cudaError_t e = optin_smem(k_gather_flat<T, D, KV>, 0, have, true);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_gather<T, D, KV>, dim3(MAXS, p.B * p.Hq), dim3(NT), 0, s, p);
+  const long long most = (long long)BH * p.gat_slots, cap = (long long)VATTN_GATHER_CTAS * device_sm_count();
+  return launch_pdl(k_gather_flat<T, D, KV>, dim3((unsigned)(most < cap ? most : cap)), dim3(NT), 0, s, p);
 }
 
 cudaError_t launch_gather(const Prob& p, cudaStream_t s) {

@@ -678,8 +678,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
         if (!all) {
           path |= 2;
           for (int c = warp; c < nbt; c += NWARP) {
-            const T* row = reinterpret_cast<const T*>(row_at(p, head_rows<T>(p, p.kc, g), row_idx(sm.vtab[c])));
-            const double s64 = score64_warp<T, D>(row, qrow, p.scale);
+            const double s64 = score64_warp<T, D>(row_ptr<T>(p, p.kc, b, g, sm.vtab[c]), qrow, p.scale);
             if (lane == 0) sm.band_s[c] = s64;
           }
           __syncthreads();

@@ -338,7 +338,7 @@ __device__ __noinline__ void head_budget(const Prob& p, int b, int h, int bh, in
   }
 }
 
-template <typename T, int D>
+template <typename T, int D, bool SPLIT>
 __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p) {
   constexpr int EPL = Elem<T>::EPL, LPR = D / EPL, RPI = 32 / LPR;
   constexpr int NE = D + 3;               // det CTA: N_f[D], D_f;  base CTA: Sr[D], Sw, Sww, Srr
@@ -459,8 +459,8 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
   if (work && base_cta && r_begin < r_end) {
     // the pivot (the first base-sample row): every CTA of the head computes the same numbers
     uint4 pk[UN];
-    pk[0] = __ldg(reinterpret_cast<const uint4*>(row_at(p, kb, word_piv)));
-    const uint4 pv = __ldg(reinterpret_cast<const uint4*>(row_at(p, vb, word_piv)));
+    pk[0] = __ldg(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, word_piv)));
+    const uint4 pv = __ldg(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, vb, word_piv)));
 #pragma unroll
     for (int u = 1; u < UN; ++u) pk[u] = pk[0];
     double w4[UN];
@@ -517,10 +517,10 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
       if (k < nbat) {
         const int4 id = *reinterpret_cast<const int4*>(s_idx + k * CB + first);
         uint4 (&dst)[UN][32] = sm.ring[warp][k & 1][kv];
-        cp_async16(&dst[0][lane], row_at(p, base, id.x));
-        cp_async16(&dst[1][lane], row_at(p, base, id.y));
-        cp_async16(&dst[2][lane], row_at(p, base, id.z));
-        cp_async16(&dst[3][lane], row_at(p, base, id.w));
+        cp_async16(&dst[0][lane], row_at<SPLIT>(p, base, id.x));
+        cp_async16(&dst[1][lane], row_at<SPLIT>(p, base, id.y));
+        cp_async16(&dst[2][lane], row_at<SPLIT>(p, base, id.z));
+        cp_async16(&dst[3][lane], row_at<SPLIT>(p, base, id.w));
       }
       cp_async_commit();
     };
@@ -636,13 +636,17 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
 
 }  // namespace
 
-template <typename T, int D>
-static cudaError_t launch_stats_t(const Prob& p, cudaStream_t s) {
+template <typename T, int D, bool SPLIT>
+static cudaError_t launch_stats_n(const Prob& p, cudaStream_t s) {
   static size_t have[VATTN_MAXDEV];
-  cudaError_t e = optin_smem(k_stats<T, D>, 0, have, true);
+  cudaError_t e = optin_smem(k_stats<T, D, SPLIT>, 0, have, true);
   if (e != cudaSuccess) return e;
   const dim3 grid(p.stat_splits > p.stat_splits_base ? p.stat_splits : p.stat_splits_base, p.Hq, 2 * p.B);
-  return launch_pdl(k_stats<T, D>, grid, dim3(NT), 0, s, p);
+  return launch_pdl(k_stats<T, D, SPLIT>, grid, dim3(NT), 0, s, p);
+}
+template <typename T, int D>
+static cudaError_t launch_stats_t(const Prob& p, cudaStream_t s) {
+  return p.row_unit == 0u ? launch_stats_n<T, D, true>(p, s) : launch_stats_n<T, D, false>(p, s);
 }
 
 cudaError_t launch_stats(const Prob& p, cudaStream_t s) {

@@ -74,8 +74,11 @@ struct Prob {
   int max_blocks, num_blocks, max_seq_len, npad, nwords;   // npad: max_seq_len rounded up to 32; nwords = npad/32
   long long sb, sh, st;                                      // KV strides in elements
   // A token's row inside a KV head's part of a cache as ONE 32-bit index, so that its address is one multiply-add:
-  // row_unit bytes * (page * row_pg + token % 16 * row_tk); row_unit = gcd of the page and token strides in bytes
+  // row_unit bytes * (page * row_pg + token % 16 * row_tk); row_unit = gcd of the page and token strides in bytes.
+  // row_unit 0: the cache, or the caller's bound on its page numbers, has more such units than 2^32; the index is then
+  // page * 16 + token % 16
   unsigned row_unit, row_pg, row_tk;
+  long long page_bytes, token_bytes;
   const void* q; const void* kc; const void* vc; const int* bt; const int* seq_lens; void* out;
   int sink, window, k;
   float topk_frac, base_rate, scale;
@@ -230,7 +233,9 @@ __device__ __forceinline__ const T* row_ptr(const Prob& p, const void* cache, in
 __device__ __forceinline__ int row_of(const Prob& p, int page, int tok) {
   return (int)((unsigned)page * p.row_pg + (unsigned)(tok & (VATTN_BLOCK - 1)) * p.row_tk);
 }
+template <bool SPLIT>                       // (kernels for caches with row_unit 0 are built apart: testing it here costs 2 % of a step)
 __device__ __forceinline__ const char* row_at(const Prob& p, const char* base, int idx) {
+  if (SPLIT) return base + (long long)((unsigned)idx / VATTN_BLOCK) * p.page_bytes + (long long)(idx & (VATTN_BLOCK - 1)) * p.token_bytes;
   return base + (unsigned long long)(unsigned)idx * p.row_unit;
 }
 // base of KV head g's rows

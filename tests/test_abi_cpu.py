@@ -61,6 +61,15 @@ def test_plan_create_validates_shape():
     rc, h = create(batch=4000, dtype=vb.DTYPE_FP32)
     assert rc == vb.OK
     vb.lib().vattn_plan_destroy(h)
+    # any bound on the page numbers, and strides that share nothing beyond the 16 bytes of their alignment
+    rc, h = create(num_blocks=2 ** 31 - 1)
+    assert rc == vb.OK
+    vb.lib().vattn_plan_destroy(h)
+    s = shape(num_blocks=2 ** 31 - 1)
+    s.kv_stride_block, s.kv_stride_head, s.kv_stride_token = 2 * 16 * 136 + 8, 16 * 136, 136
+    h = C.c_void_p()
+    assert vb.lib().vattn_plan_create(C.byref(s), C.byref(h)) == vb.OK
+    vb.lib().vattn_plan_destroy(h)
     assert vb.lib().vattn_plan_create(None, None) == vb.ERR_INVALID_ARG
 
 

@@ -163,3 +163,37 @@ def test_plans_that_take_turns_on_one_workspace():
     del plans[1]                                                     # (its counters are still lying there)
     run(0, False)
     run(0, True)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("padded", [False, True])
+def test_cache_that_a_32_bit_row_index_does_not_cover(dtype, padded):
+    # such plans were refused: a bound on the page numbers that bounds nothing (2^31 - 1), and page and token strides whose
+    # common divisor is the 16 bytes of their alignment
+    import torch
+    from helpers import assert_parity, run_gpu, run_oracle
+    from paper_2510_05688_b200 import binding as vb
+    from paper_2510_05688_b200 import synth
+    Hq, Hkv, d = 8, 2, 64
+    case = synth.make_case("rows", dtype=dtype, B=2, Hq=Hq, Hkv=Hkv, d=d, seq_lens=[3000, 129], sink=4, window=8, k=100, eps=0.05,
+                           delta=0.05, seed=5, gen_seed=6, heavy=dict(R=12, c1=5.0, alpha=(0.75, 1.25)), params=dict(base_rate=0.05))
+    dev, nblk = vb.case_to_device(case), case.num_blocks
+    strides = (0, 0, 0)
+    if padded:
+        align = 8 if dtype == "bf16" else 4
+        st = d + align
+        sh = 16 * st
+        strides = (Hkv * sh + align, sh, st)
+        assert np.gcd(strides[0], st) == align
+        for name in ("k_cache", "v_cache"):
+            buf = torch.full((nblk * strides[0],), 7.0, dtype=dev[name].dtype, device="cuda")
+            torch.as_strided(buf, (nblk, Hkv, 16, d), (*strides, 1)).copy_(dev[name])
+            dev[name] = buf
+    plan = vb.Plan(batch=2, num_q_heads=Hq, num_kv_heads=Hkv, head_dim=d, max_blocks_per_seq=case.max_blocks_per_seq,
+                   num_blocks=2 ** 31 - 1, max_seq_len=case.max_blocks_per_seq * 16, kv_strides=strides,
+                   dtype=vb.DTYPE_BF16 if dtype == "bf16" else vb.DTYPE_FP32)
+    for mode in (dict(), dict(gather_mode=1)):
+        out_ref, det = run_oracle(case, **mode)
+        got, dbg, _ = run_gpu(case, plan=plan, dev=dev, **mode)
+        assert_parity(case, got, dbg, det, out_ref)
+    assert plan.last_status() == 0
