@@ -233,12 +233,12 @@ __device__ __noinline__ Found select_general(const Prob& p, unsigned char* smem,
   // requested at a time
   auto for_slice = [&](auto f) {
 #pragma unroll 1
-    for (int u0 = 0; u0 < PT; u0 += 4) {
-      float s[4];
+    for (int u0 = 0; u0 < PT; u0 += 1) {
+      float s[1];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) { const int i = s0 + tid + NT * (u0 + e); s[e] = i < l_start ? __ldg(sc + i) : 0.f; }
+      for (int e = 0; e < 1; ++e) { const int i = s0 + tid + NT * (u0 + e); s[e] = i < l_start ? __ldg(sc + i) : 0.f; }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
+      for (int e = 0; e < 1; ++e) {
         const int u = u0 + e, i = s0 + tid + NT * u;
         if (u >= PT) break;
         const bool v = i < l_start;
@@ -255,7 +255,14 @@ __device__ __noinline__ Found select_general(const Prob& p, unsigned char* smem,
   else {
     int need_eq;
     const unsigned Tk = radix_select<NT, unsigned>(sm, kk, need_eq, [&](auto body) {
-      for_slice([&](int, int, bool v, unsigned key) { if (v) body(key); });
+#pragma unroll 1
+      for (int i0 = s0 + tid; i0 < l_start; i0 += 4 * NT) {      // (four scores requested at a time)
+        float s[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] = i0 + e * NT < l_start ? __ldg(sc + i0 + e * NT) : 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) if (i0 + e * NT < l_start) body(~ord_f32(s[e] == s[e] ? s[e] : -CUDART_INF_F));
+      }
     });
     const float Tf = unord_f32(~Tk);
     hi = __fadd_ru(Tf, 2.f * gamma); lo = __fadd_rd(Tf, -2.f * gamma);
@@ -456,12 +463,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
   int path = 0;
   float hi = CUDART_INF_F, lo = CUDART_INF_F;          // members: s > hi; near-tie band: lo <= s <= hi
   int nbt = 0, band_mode = 0;
-  // There is a threshold to find, and the list is likely to hold what the bound lets through (see sel_cap in api.cu).  A
-  // top-k set of a tenth of 131,071 tokens mostly overflows it: 622 us per step of 32 heads when that was found out only
-  // after the compare pass, 600 like this, and 522 with the general case's scores requested four at a time.
-  const int stride = sample_stride(n, SAMPLES);
-  const float through = (float)kk + 4.f * __fsqrt_rn((float)kk * (float)stride) + 9.f * (float)stride;
-  const bool usual = kk > 0 && kk < mlen && (mlen <= cap || through + 2.f * __fsqrt_rn(through * (float)stride) <= (float)cap);
+  // there is a threshold to find, and the list is likely to hold what the bound lets through (see sel_kmax in api.cu)
+  const bool usual = kk > 0 && kk < mlen && (mlen <= cap || kk <= p.sel_kmax);
   bool general = kk > 0 && !usual;
   if (!usual && warp == NWARP - 1 && lane == 0)
     sm.gamma[0] = __double2float_ru(gfac * (double)__uint_as_float(kmax_bits));
@@ -484,7 +487,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
     // against one another took 106 instead of 72 us per step at 32 heads x 32,768 tokens with logits around 20, and 780 instead
     // of 176 at 131,071.)
     if (mlen > cap) {
-      const int ns_all = (n + stride - 1) / stride;
+      const int stride = sample_stride(n, SAMPLES), ns_all = (n + stride - 1) / stride;
       unsigned kept[SAMPLES / NT];             // (all ones: not a middle token)
 #pragma unroll
       for (int e = 0; e < SAMPLES / NT; ++e) {

@@ -93,6 +93,7 @@ struct Prob {
   float* scores;          // [B,Hq,npad]
   unsigned* m_ord;        // [B,Hq]  order-preserving encoding of the running max score
   int sel_cap;            // candidates of I_t that a selection CTA holds; heads with no more middle tokens need no bound
+  int sel_kmax;           // larger top-k sets (of more middle tokens than that list holds) take the general selection at once
   unsigned* kabsmax;      // [B,Hkv] bits of max |K element| over the sequence
   unsigned* unit_ctr;     // [1] work-unit counter of the persistent score kernel
   unsigned* tickets;      // [B,Hq] "last CTA done" counters of the dense kernel
