@@ -103,13 +103,14 @@ typedef struct {
   double  *stats;                 /* [B,Hq,8] D_f, sigma^2, Tr(Sigma), D_hat, |N_hat|_2, n_s, b0, m (weights are
                                      exp(s - m) with m the head's largest fp32 score) */
   float   *scores;                /* [B,Hq,cap] fp32 scores s_i = scale * <K[i], q> */
-  int32_t *paths;                 /* [B,Hq] which code path the top-k selection took: bit 0 the usual one (a
-                                     bound from a sample, then an exact selection among the tokens above it; bit 4
-                                     instead of bit 0 beyond 131,072 tokens; neither: the radix select over the whole
-                                     middle range), bit 1
-                                     near-tie tokens were rescored in fp64 and ranked from a list, bit 2 they were
-                                     too many for the list and the exact 64-bit radix select ran
-                                     (VATTN_STATUS_BAND_OVERFLOW) */
+  int32_t *paths;                 /* [B,Hq] which code path the top-k selection took: bit 0 the usual one (a bound from every
+                                     32nd token's score where there are many, then an exact selection among the tokens
+                                     above it), bit 4 instead of bit 0 where the bound came from fewer tokens (every 64th,
+                                     128th, ...: contexts above 131,072 tokens, above 65,536 or 32,768 with many heads);
+                                     neither: the radix select over the whole middle range (every middle token selected, or
+                                     more candidates than the list holds); bit 1 near-tie tokens were rescored in fp64 and
+                                     ranked from a list, bit 2 they were too many for the list and the exact 64-bit radix
+                                     select ran (VATTN_STATUS_BAND_OVERFLOW) */
   unsigned long long *kernel_ticks; /* [VATTN_NUM_TICKS][2] device-side time stamps in ns (%globaltimer): rows 1-5
                                      the score kernel, the walk kernel, the selection kernel, the statistics kernel and
                                      the gather kernel, row 0 unused ([k][0] = earliest CTA start,

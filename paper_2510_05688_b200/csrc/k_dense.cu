@@ -617,7 +617,8 @@ extern "C" int vattn_dense_decode_noalloc(const vattn_shape* shape, float scale,
   if (bits & 15) return VATTN_ERR_INVALID_ARG;
   if (!(scale == scale) || isinf(scale)) return VATTN_ERR_INVALID_ARG;
 
-  // layout inside the fixed array: status word | tickets (must start at zero) | split partials
+  // layout inside the fixed array: status word | tickets (must start at zero; room for three per head, which the header's
+  // limit on the problem counts, one is used) | split partials
   const size_t BH = (size_t)s.batch * s.num_q_heads, D = (size_t)s.head_dim;
   const int G = s.num_q_heads / s.num_kv_heads, GC = (G + 3) / 4;
   const size_t groups = (size_t)s.batch * s.num_kv_heads * GC;

@@ -9,15 +9,16 @@
 // at large batch, how many heads an SM works on at once; so it keeps little in shared memory and in registers, reads
 // the scores where they are (L2), and takes few phases:
 //   A  a lower bound of the k-th largest score from a sample (every 32nd token): the sample's key of rank
-//      rs + 4 sqrt(rs) + 8, rs = k * samples / |M|, four standard deviations below where rank k is expected;
+//      rs + 4 sqrt(rs) + 9, rs = k * samples / |M|, four standard deviations below where rank k is expected (one histogram
+//      of the top 12 key bits, a second one of the next 12 where the bin is crowded);
 //   B  every score is compared with it: the candidates, one and a half times k or so, go to a list in an order that
 //      depends on the data only (thread order, one prefix sum);
 //   C  the exact rank-k key T among the candidates: a 12-bit histogram, then the few keys of the bin ranked directly.
 // The stored scores differ from the exact inner products by at most gamma (a bound from the summation structure
 // of the score kernel), so candidates above T + 2 gamma are certainly selected, candidates below T - 2 gamma
 // certainly not, and the few in between are rescored in fp64 from their K rows and ranked exactly.
-// Anything unusual (fewer than k candidates, too many candidates or near-ties, every middle token selected) takes
-// the general path: a 32-bit radix select over the whole range with re-read scores, and for more than 1,024 near-ties
+// Anything unusual (fewer than k candidates, too many candidates or near-ties, a k too large for the list, every middle
+// token selected) takes the general path: a 32-bit radix select over the whole range with re-read scores, and for more than 1,024 near-ties
 // (constant keys, a zero query) an exact 64-bit radix select over fp64 scores.
 // (A version with one 1024-thread CTA per head that held all keys in 227 KB of shared memory: 193 us instead of 95 at
 // 1,024 heads of 4,096 to 32,768 tokens, 55 instead of 35 at 256 heads of 32,768, 45 instead of 23 at 256 heads of
@@ -205,7 +206,7 @@ __device__ __noinline__ double score64_thread(const T* krow, const T* qrow, floa
 }
 
 // "I_t is written and marked in the base sample's walk array" (thread 0, behind a barrier): one cumulative fence, then
-// both words of the head
+// both words of the head, which are stored together
 __device__ __forceinline__ void publish(const Prob& p, int bh, unsigned long long word) {
   __threadfence();
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&p.words[bh].sample), "l"(word) : "memory");
@@ -436,8 +437,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
     const double roundings = (p.dtype == VATTN_DTYPE_BF16) ? 512.0 : 16.0;
     gfac = roundings * 5.9604644775390625e-8 * fabs((double)p.scale) * sa * 1.000001;
   }
-  // the first entries of the head's list of marked positions are read unconditionally by the budget: "none" until set
-  if (tid < 256) p.hole_pos[(long long)bh * 2 * VATTN_BANDCAP + tid] = 0x7FFFFFFF;
   int* wa0 = p.walk_tok + (long long)bh * 4 * p.npad;            // base sample's walk: tokens (row indices at + npad)
   int* wa1 = wa0 + 2 * p.npad;                                   // final sample's walk
   const int W0 = walk_region(n_s > 0 ? b0 : 0, n_s, mlen, kk);   // entries the walk kernel wrote
@@ -703,7 +702,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
             sm.vtab[c] = tok | (int)0x80000000;
           }
         }
-        path |= n <= 131072 ? 1 : 16;
+        path |= mlen <= cap || n <= 32 * SAMPLES ? 1 : 16;       // (16: a bound from fewer tokens than every 32nd)
       }
       __syncthreads();
     }

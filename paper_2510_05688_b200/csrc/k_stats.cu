@@ -9,8 +9,8 @@
 //     sigma^2, Tr(Sigma), D_hat, |N_hat|,  b_D, b_N, b_SDPA,  b = clamp(ceil(b_X), b0, n_s)
 // in fp64 (the two square-root / division chains on two lanes, the 15 split points of b_SDPA on 15 lanes).  Heads
 // whose I_dyn is a prefix of the part of the walk that the selection kernel listed (the usual case) are then done;
-// for the others the same CTA lists the rest of the final sample (Algorithm 1 line 7): it continues the walk from
-// where the list ends, or, when b is the whole residual, lists every residual token in token order.
+// for the others the same CTA lists the final sample (Algorithm 1 line 7): the laid-out entries of its walk without the
+// marked ones, then further positions, or, when b is the whole residual, every residual token in token order.
 //
 // Everything that decides the integer budget is fp64: the same inputs must give the same ceil() as a
 // plain fp64 evaluation.  Variances are accumulated around a pivot (the first base-sample row), which
@@ -355,8 +355,7 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
   __shared__ double pivT[D];             // the pivot's w*V, element-major per lane: pivT[e * LPR + j]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // grid (S, Hq, 2 B): the deterministic-row CTAs of every head come first in dispatch order (their word is
-  // published first), the base-row CTAs follow
+  // grid (S, Hq, 2 B): the deterministic-row CTAs of every head come first in dispatch order, the base-row CTAs follow
   const bool base_cta = (int)blockIdx.z >= p.B;
   const int h = blockIdx.y, b = base_cta ? blockIdx.z - p.B : blockIdx.z, g = h / p.G;
   const int bh = b * p.Hq + h;
@@ -387,8 +386,8 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
   __shared__ unsigned long long s_word;
   __shared__ int s_flag;
   __shared__ int s_misc[8];
-  // deterministic-row CTAs wait for "the list of I_t is written" (a 32-bit word, published first), base-row CTAs
-  // for the 64-bit word
+  // deterministic-row CTAs wait for a 32-bit word of their own, base-row CTAs for the 64-bit one (the selection kernel
+  // stores both together, once I_t is marked in the base walk)
   HeadWords* hw = p.words + bh;
   if (tid == 0) {
     const unsigned long long v = base_cta ? wait_word64(&hw->sample, VATTN_WORD_SPINS)

@@ -29,15 +29,13 @@ struct HeadMeta {
   int band_mode;    // 1: the near-ties were too many for the list; their verdicts are bits of the bitmap
   float m;          // largest fp32 score of the head (softmax stabiliser)
   float hi, lo;     // a middle token is in I_t if its score is above hi; scores in [lo, hi] are near-ties
-  int pad0;
   int dyn_listed;   // budgets up to this many are served as "the non-members among the first J positions of the final
   int dyn_J;        //   sample's walk" (dyn_J positions are in the walk array, members marked), larger ones from a list
   int path;         // code path of the selection (vattn_debug.paths)
-  int pad2;
   int base_J;       // the base sample = the unmarked entries among the first base_J of its walk array
   int holes2;       // members of I_t at positions of the final sample's walk beyond its array (hole_pos + BANDCAP)
-  int pad1;
   int holes1;       // marked entries among the first dyn_J of the final sample's walk (their positions in hole_pos)
+  int pad[3];
 };
 
 // What the gather kernel needs of a head (published by the statistics kernel, see publish_budget).
@@ -53,7 +51,7 @@ struct GMeta { int b, n_s; float m; int n, L, list, W1, start; };
 struct __align__(256) HeadWords {
   unsigned long long sample;  // selection -> statistics, base rows: I_t is written and marked in the base sample's walk array:
                               //   2 | (some K element is not finite) << 2 | base_J << 3 | row index of the pivot << 32
-  unsigned topk;              // selection -> statistics, deterministic rows: "the list of I_t is written": 1 | K not finite << 1
+  unsigned topk;              // selection -> statistics, deterministic rows: 1 | K not finite << 1 (stored with `sample`)
   unsigned pad0;
   unsigned long long budget[2];   // statistics -> gather: the head's GMeta, packed (one 16-byte word)
   int start;                  // ... and its `start`, where that is not zero
@@ -100,7 +98,7 @@ struct Prob {
   HeadWords* words;       // [B,Hq] words through which the step's kernels hand over and count
   unsigned* status;       // [1]
   unsigned* bitmap;       // [B,Hq,nwords] near-tie tokens that made it into I_t (used when they are too many for a list)
-  int* vtab;              // [B,Hq,BANDCAP] near-tie tokens ascending, bit 31 = member of I_t
+  int* vtab;              // [B,Hq,BANDCAP] near-tie tokens, in no particular order; bit 31 = member of I_t
   int* topk_idx;          // [B,Hq,2,npad] I_t; then the row indices (row_of) of I_f: sink, I_t, window
   int* sel_cnt;           // [B,Hq,2,npad/16+32] ordered counts of the selection's general path
   int* walk_tok;          // [B,Hq,2,2,npad] the first positions of both walks (computed beside the score pass): per
@@ -108,8 +106,7 @@ struct Prob {
                           //   of I_t (token = -1; the row index stays valid): a sample is the unmarked entries of a prefix
   unsigned* wkeys;        // [B,Hq,8] round keys of the final sample's walk (for the gather kernel's array extension)
   int* hole_pos;          // [B,Hq,2,VATTN_BANDCAP] positions of the marked entries of the final sample's walk array, in
-                          //   no particular order (the first 256 words read INT_MAX where there is none); then the
-                          //   positions of the members of I_t beyond the array
+                          //   no particular order; then the positions of the members of I_t beyond the array (counts: HeadMeta)
   int* dyn_idx;           // [B,Hq,3,npad] I_dyn as a list (tokens, row indices) for budgets beyond the walk arrays
                           //               (scratch of the near-tie overflow path while the selection runs)
   HeadMeta* meta;         // [B,Hq]

@@ -195,3 +195,14 @@ def test_block_sizes_of_the_selection(B, Hq, tokens):
     # decides, whatever the sequences are now)
     lens = [(389 * i) % 3000 + 1 for i in range(B)]
     check(small("bf16", lens, Hq=Hq, Hkv=1, d=64, k=60, max_blocks=tokens // 16))
+
+
+def test_paths_tell_where_the_bound_came_from():
+    # 75 heads on a plan for up to 65,536 tokens run 512 threads (every 32nd token up to there); 1 head runs 1,024
+    lens = [700] * 14 + [65536]
+    _, dbg, plan = run_gpu(small("bf16", lens, Hq=5, Hkv=1, d=64, k=100))
+    assert (dbg["paths"] & 17 == 1).all() and plan.last_status() == 0
+    _, dbg, plan = run_gpu(small("bf16", [700] * 148 + [70000], Hq=1, Hkv=1, d=64, k=100))       # (149 heads: 512 threads)
+    assert (dbg["paths"][:148] & 17 == 1).all() and (dbg["paths"][148] & 17 == 16).all()
+    _, dbg, plan = run_gpu(small("bf16", [700, 70000], Hq=1, Hkv=1, d=64, k=100))
+    assert (dbg["paths"] & 17 == 1).all()
