@@ -119,14 +119,76 @@ __device__ __forceinline__ int block_scan_reg(int val, int* wtot, int& total) {
 // CTAs that share `rows` rows: a share of less than stat_rows does not pay for a CTA's fixed costs
 __device__ __forceinline__ int stat_ctas(int rows, int most, int share) { return min(most, max(1, (rows + share - 1) / share)); }
 
+// I_dyn as a list: budgets beyond what the known positions serve (unusual: saturated budgets), and for the debug buffer
+__device__ __noinline__ void list_sample(const Prob& p, int b, int h, int bh, int bfin, int J, bool listed, int* misc) {
+  const HeadMeta mt = ld_meta(p.meta + bh);
+  const int tid = threadIdx.x, n_s = mt.n_s, b0 = mt.b0;
+  int* dl = p.dyn_idx + (long long)bh * 3 * p.npad;
+  if (listed || (p.dbg.dyn_idx && bfin > 0)) {
+    __shared__ unsigned rkeys[8];
+    if (tid < 2) walk_keys(p, b, h, 1, tid, rkeys);
+    __syncthreads();
+    const int s0 = mt.s0, l_start = mt.l_start;
+    const int* vt = p.vtab + (long long)bh * VATTN_BANDCAP;
+    const float* sc = p.scores + (long long)bh * p.npad;
+    const unsigned* gbitmap = p.bitmap + (long long)bh * p.nwords;
+    const bool whole = bfin >= n_s;                    // every residual token, in token order
+    const Walk wk = make_walk(rkeys, l_start - s0);
+    // the walk's laid-out entries are read, not computed again (522 -> 438 us per step of 32 heads x 131,071 tokens, a tenth of
+    // them top-k; 1,165 -> 763 at 64 x 65,536 with nearly all of them read)
+    const int W1 = walk_region(dyn_listed_want(p, n_s, b0), n_s, l_start - s0, mt.kk);
+    const int* wt = p.walk_tok + ((long long)bh * 4 + 2) * p.npad;
+    int have = 0;
+    int cur = whole ? s0 : 0;
+    const int end = whole ? l_start : (l_start - s0);
+#pragma unroll 1
+    while (have < bfin && cur < end) {
+      int tokc[WPT];
+      int nres = 0;
+#pragma unroll
+      for (int q_ = 0; q_ < WPT; ++q_) {
+        tokc[q_] = -1;
+        const int x = cur + tid * WPT + q_;
+        if (x < end) {
+          const bool laid = !whole && x < W1;          // (an entry of the array: marked if it is a member)
+          const int tok = whole ? x : laid ? __ldcg(wt + x) : s0 + walk_at(wk, x);
+          if (laid ? tok >= 0 : !in_topk(mt, vt, gbitmap, tok, __ldg(sc + tok))) { tokc[q_] = tok; ++nres; }
+        }
+      }
+      int tot1;
+      int rank = have + block_scan_reg(nres, misc, tot1);
+#pragma unroll
+      for (int q_ = 0; q_ < WPT; ++q_) {
+        if (tokc[q_] >= 0) {
+          if (rank < bfin) { dl[rank] = tokc[q_]; dl[p.npad + rank] = row_of(p, page_of(p, b, tokc[q_] >> 4), tokc[q_]); }
+          ++rank;
+        }
+      }
+      have += tot1;
+      cur += NT * WPT;
+    }
+  }
+  if (listed) {                                        // a listed head: its list is complete now
+    __syncthreads();
+    if (tid == 0) publish_budget(p, bh, GMeta{bfin, n_s, mt.m, 1, J, 1, mt.dyn_J, 0});
+  }
+  if (p.dbg.dyn_idx) {
+    __syncthreads();
+    int* dbg = p.dbg.dyn_idx + (long long)bh * p.max_seq_len;
+    for (int i = tid; i < bfin; i += NT) dbg[i] = __ldcg(dl + i);
+  }
+}
+
 // Budget of head bh from the partials of its S0 + S1 CTAs, by the last of them.  It stands between the rows and the
 // gather of every head, so it is a short chain: everything it reads is requested at once (one round trip), thread e
 // adds element e of both kinds in split order, warp k the k-th scalar sum, one barrier, and every warp evaluates the
 // budgets for itself (no broadcast).  What does not depend on the rows is computed elsewhere: coefficients on the
 // host, pre[0..2] = n_s / b0, 1 / b0, 1 / (b0 - 1) before the CTA's waits.  scal: 16 doubles and 2 NWARP ints of shared memory.
-// (7 us from a head's last row to its published budget before, one head of 1,024 tokens.)
+// (7 us from a head's last row to its published budget before, one head of 1,024 tokens.)  Inlined into the kernel, so that
+// the parameters are constants of the launch: as a function of its own it read each of them through memory, and the chain
+// took 5.0 instead of 3.8 us at 32 heads x 32,768 tokens; only the list is one.
 template <int D>
-__device__ __noinline__ void head_budget(const Prob& p, int b, int h, int bh, int S0, int S1, const double* pre, double* scal, int* misc) {
+__device__ __forceinline__ void head_budget(const Prob& p, int b, int h, int bh, int S0, int S1, const double* pre, double* scal, int* misc) {
   constexpr int NE = D + 3;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double* src = p.stat_part + (long long)bh * 2 * MAXS * NE;
@@ -281,61 +343,7 @@ __device__ __noinline__ void head_budget(const Prob& p, int b, int h, int bh, in
     __syncthreads();
     if (tid == 0 && !listed) publish_budget(p, bh, GMeta{bfin, n_s, mt.m, 1, J, 0, mt.dyn_J, start});      // (a listed head: when its list is complete)
   }
-  int* dl = p.dyn_idx + (long long)bh * 3 * p.npad;
-  // ---- I_dyn as a list: budgets beyond the walk array (unusual: saturated budgets), and for the debug buffer
-  if (listed || (p.dbg.dyn_idx && bfin > 0)) {
-    __shared__ unsigned rkeys[8];
-    if (tid < 2) walk_keys(p, b, h, 1, tid, rkeys);
-    __syncthreads();
-    const int s0 = mt.s0, l_start = mt.l_start;
-    const int* vt = p.vtab + (long long)bh * VATTN_BANDCAP;
-    const float* sc = p.scores + (long long)bh * p.npad;
-    const unsigned* gbitmap = p.bitmap + (long long)bh * p.nwords;
-    const bool whole = bfin >= n_s;                    // every residual token, in token order
-    const Walk wk = make_walk(rkeys, l_start - s0);
-    // the walk's laid-out entries are read, not computed again (522 -> 438 us per step of 32 heads x 131,071 tokens, a tenth of
-    // them top-k; 1,165 -> 763 at 64 x 65,536 with nearly all of them read)
-    const int W1 = walk_region(dyn_listed_want(p, n_s, b0), n_s, l_start - s0, mt.kk);
-    const int* wt = p.walk_tok + ((long long)bh * 4 + 2) * p.npad;
-    int have = 0;
-    int cur = whole ? s0 : 0;
-    const int end = whole ? l_start : (l_start - s0);
-#pragma unroll 1
-    while (have < bfin && cur < end) {
-      int tokc[WPT];
-      int nres = 0;
-#pragma unroll
-      for (int q_ = 0; q_ < WPT; ++q_) {
-        tokc[q_] = -1;
-        const int x = cur + tid * WPT + q_;
-        if (x < end) {
-          const bool laid = !whole && x < W1;          // (an entry of the array: marked if it is a member)
-          const int tok = whole ? x : laid ? __ldcg(wt + x) : s0 + walk_at(wk, x);
-          if (laid ? tok >= 0 : !in_topk(mt, vt, gbitmap, tok, __ldg(sc + tok))) { tokc[q_] = tok; ++nres; }
-        }
-      }
-      int tot1;
-      int rank = have + block_scan_reg(nres, misc, tot1);
-#pragma unroll
-      for (int q_ = 0; q_ < WPT; ++q_) {
-        if (tokc[q_] >= 0) {
-          if (rank < bfin) { dl[rank] = tokc[q_]; dl[p.npad + rank] = row_of(p, page_of(p, b, tokc[q_] >> 4), tokc[q_]); }
-          ++rank;
-        }
-      }
-      have += tot1;
-      cur += NT * WPT;
-    }
-  }
-  if (listed) {                                        // a listed head: its list is complete now
-    __syncthreads();
-    if (tid == 0) publish_budget(p, bh, GMeta{bfin, n_s, mt.m, 1, J, 1, mt.dyn_J, 0});
-  }
-  if (p.dbg.dyn_idx) {
-    __syncthreads();
-    int* dbg = p.dbg.dyn_idx + (long long)bh * p.max_seq_len;
-    for (int i = tid; i < bfin; i += NT) dbg[i] = __ldcg(dl + i);
-  }
+  if (listed || p.dbg.dyn_idx) list_sample(p, b, h, bh, bfin, J, listed, misc);
 }
 
 template <typename T, int D, bool SPLIT>
