@@ -2,17 +2,22 @@
 //     N = N_f + (n_s/b) * sum_{I_dyn} w_i V[i],   D = D_f + (n_s/b) * sum_{I_dyn} w_i,   out = N / D
 // which is SDPA_{S,p} of Sec. 3 with p = 1 on I_f and p = b/n_s on I_dyn.
 //
-// A gather of V rows.  Work unit = a chunk of consecutive entries of one head's I_dyn, taken by a CTA in sections of SEC:
-//   1  one thread per entry: its row index (from the walk array or the list; computed for entries beyond the array and
-//      for whole-residual budgets) to shared memory;
-//   2  the first rows are requested; meanwhile, again one thread per entry, the weight expf(s - m) from the stored fp32
-//      score (no K re-read; members of I_t weigh nothing) to shared memory;
-//   3  every warp streams its rows: LPR lanes fetch one row with one 16-byte asynchronous copy each into a ring of S
-//      batches that belongs to the lane alone (a lane reads what it copied itself, so nothing is synchronised), and add
-//      weight times row.
-// What bounds it: DRAM at large batch, dependent round trips (budget, entries, rows, partials) for one sequence.
-// (A version that kept rows in registers, with entries, scores, exps and validity tests handled by the lanes of a row,
-// issued about 250 instructions per eight rows and reached half the bandwidth.)
+// A gather of V rows.  Work unit = a chunk of consecutive entries of one head's I_dyn, taken by a CTA; its warps work for
+// themselves, without barriers, each on every fourth batch of rows.  A warp takes its entries in stages of 32 (64 for short
+// bf16 rows):
+//   1  one lane per entry: token and row index (from the walk array or the list; computed for entries beyond the array and
+//      for whole-residual budgets), requested while the stage before is streamed; the row indices go to shared memory;
+//   2  again one lane per entry, the weight expf(s - m) from the stored fp32 score (no K re-read; members of I_t weigh
+//      nothing; the scores are requested three batches ahead) to shared memory;
+//   3  the rows: LPR lanes fetch one row with one 16-byte asynchronous copy each into a ring of S batches that belongs to
+//      the lane alone (a lane reads what it copied itself, so nothing is synchronised), and add weight times row.  The ring
+//      runs on from one stage to the next.
+// What bounds it: DRAM and L2 at large batch (scattered rows), dependent round trips (budget, entries, rows, partials) for
+// one sequence.
+// (Sections of 256 entries per CTA, staged between barriers, drained the ring at the end of each: 619 instead of 594 us per
+// step at 1,024 heads of 4,096 to 32,768 tokens, 205.7 instead of 202.5 at 256 x 32,768, 109.3 instead of 106.2 at 128 x
+// 32,768.  A version that kept rows in registers, with entries, scores, exps and validity tests handled by the lanes of a
+// row, issued about 250 instructions per eight rows and reached half the bandwidth.)
 // Partials are added in chunk order by the last CTA of the head ("ticket"), so results are reproducible.
 //
 // Two decompositions:
@@ -37,7 +42,6 @@ namespace {
 constexpr int NT = 128;
 constexpr int NWARP = NT / 32;
 constexpr int UN = 4;              // rows per batch of a row group
-constexpr int SEC = 256;           // entries staged at a time
 constexpr int MAXS = VATTN_GATHER_SLOTS;
 constexpr int FLAT_MAX_HEADS = VATTN_GATHER_FLAT_HEADS;
 __host__ __device__ constexpr int min_chunk(int heads) { return heads >= 512 ? 512 : heads > 160 ? 256 : 128; }   // per-head decomposition
@@ -48,17 +52,24 @@ struct Gather {
   static constexpr int EPL = Elem<T>::EPL, LPR = D / EPL, RPI = 32 / LPR, NE = D + 1;
   static constexpr int WB = RPI * UN, CB = NWARP * WB;      // rows per warp and per CTA of a batch
   static constexpr int S = 3;                               // batches in flight
-  static_assert(SEC % CB == 0 && LPR >= 8, "whole batches per section; two hand-over levels of the K+V variant");
+  static constexpr int EN = WB > 8 ? 2 : 1;                 // entries per lane of a stage ...
+  static constexpr int NB = 32 * EN / WB;                   // ... which is this many of the warp's batches
+  static_assert(NB > S && NB * WB == 32 * EN && LPR >= 8, "a stage is opened after the one before it has its weights; two hand-over levels of the K+V variant");
+  union WarpMem {
+    uint4 ring[S][UN][32];
+    float part[NE];                                         // the warp's sums, when its rows are done
+    __device__ WarpMem() {}
+  };
   struct Sm {
-    uint4 ring[NWARP][S][UN][32];
-    int idx[SEC];                                           // row indices
-    float w[SEC];                                           // weights
-    float part[NWARP][NE];
+    WarpMem warp[NWARP];
+    int idx[NWARP][2][32 * EN];                             // row indices of two stages
+    float w[NWARP][2][32 * EN];                             // weights
     unsigned keys[8];
     HeadMeta mt;
     GMeta meta;
     float den;
     int flag;
+    __device__ Sm() {}
   };
   static __device__ __forceinline__ void unpack(const uint4& r, float (&v)[EPL]) {
     if (EPL == 8) {
@@ -96,98 +107,84 @@ struct Gather {
     const float* sc = p.scores + (long long)bh * p.npad;
     const float m = meta.m;
     const int rsub = lane / LPR, j = lane % LPR;
-    const int mine = warp * WB + rsub * UN;                 // this row group's first row of a batch
     const char* vb = head_rows<T>(p, p.vc, g) + j * 16;
     float acc[EPL], dd = 0.f;
 #pragma unroll
     for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
 
-#pragma unroll 1
-    for (int x0 = r_begin; x0 < r_end; x0 += SEC) {
-      const int cnt = min(SEC, r_end - x0), nbat = (cnt + CB - 1) / CB;
-      __syncthreads();                                      // the section before this one (or the chunk) has been used
-      // ---- 1: row indices (the padding of the last batch repeats a real row)
-      int tok[SEC / NT];
-      if (x0 + cnt <= W1) {
+    // Every warp works for itself, without a barrier.  Its share of the chunk (WB of every CB entries) is taken in stages
+    // of 32 EN entries: a stage is opened (its row indices go to shared memory, its scores and the next stage's entries are
+    // requested) when its first rows are wanted, S batches before its weights are.
+    const int nbat = (r_end - r_begin + CB - 1) / CB;
+    int tok_n[EN], row_n[EN];                               // the next stage's entries
+    float sc_n[EN];                                         // the open stage's scores
+    int tok_o[EN];                                          // ... and tokens (-1: weighs nothing)
+    auto entry = [&](int t, int i) { const int at = i * 32 + lane; return r_begin + (t * NB + at / WB) * CB + warp * WB + at % WB; };
+    auto load = [&](int t) {
 #pragma unroll
-        for (int i = 0; i < SEC / NT; ++i) {
-          const int x = x0 + min(i * NT + tid, cnt - 1);
-          tok[i] = __ldcg(dyn + x);
-          sm.idx[i * NT + tid] = __ldcg(drow + x);
-        }
-      } else {
-        if (ident) {
-#pragma unroll
-          for (int i = 0; i < SEC / NT; ++i) tok[i] = sm.mt.s0 + x0 + min(i * NT + tid, cnt - 1);
-        } else {
-          // cycle walking repeats the network until the value falls below |M|: a thread goes on to its next entry as
-          // soon as one is finished instead of waiting for its warp's slowest lane
-          const Walk wk = make_walk(sm.keys, sm.mt.l_start - sm.mt.s0);
-          int i = 0;
-          unsigned cur = (unsigned)(x0 + min(tid, cnt - 1));
-          while (i < SEC / NT) {
-            cur = walk_pass(wk, cur);
-            if (cur < wk.mlen) {
-              sm.idx[i * NT + tid] = sm.mt.s0 + (int)cur;
-              ++i;
-              cur = (unsigned)(x0 + min(i * NT + tid, cnt - 1));
-            }
-          }
-#pragma unroll
-          for (i = 0; i < SEC / NT; ++i) tok[i] = sm.idx[i * NT + tid];
-        }
-#pragma unroll
-        for (int i = 0; i < SEC / NT; ++i) {
-          const int x = x0 + min(i * NT + tid, cnt - 1);
-          if (x < W1) { tok[i] = __ldcg(dyn + x); sm.idx[i * NT + tid] = __ldcg(drow + x); }
-          else sm.idx[i * NT + tid] = row_of(p, page_of(p, b, tok[i] >> 4), tok[i]);
+      for (int i = 0; i < EN; ++i) {
+        const int x = min(entry(t, i), r_end - 1);          // (the padding of the last batch repeats a real row)
+        if (x < W1) { tok_n[i] = __ldcg(dyn + x); row_n[i] = __ldcg(drow + x); }
+        else {
+          tok_n[i] = sm.mt.s0 + (ident ? x : walk_at(make_walk(sm.keys, sm.mt.l_start - sm.mt.s0), x));
+          row_n[i] = row_of(p, page_of(p, b, tok_n[i] >> 4), tok_n[i]);
         }
       }
-      __syncthreads();
-      // ---- the first rows
-      auto issue = [&](int k, int slot_) {                  // batch k into a slot of the ring
-        if (k < nbat) {
-          const int4 id = *reinterpret_cast<const int4*>(sm.idx + k * CB + mine);
-          uint4 (&dst)[UN][32] = sm.ring[warp][slot_];
-          cp_async16(&dst[0][lane], row_at<SPLIT>(p, vb, id.x));
-          cp_async16(&dst[1][lane], row_at<SPLIT>(p, vb, id.y));
-          cp_async16(&dst[2][lane], row_at<SPLIT>(p, vb, id.z));
-          cp_async16(&dst[3][lane], row_at<SPLIT>(p, vb, id.w));
-        }
-        cp_async_commit();
-      };
+    };
+    auto open = [&](int t) {
 #pragma unroll
-      for (int k = 0; k < S; ++k) issue(k, k);
-      if (KV) dots(p, sm, bh, nbat, mine);                  // (K+V variant) the scores, from the K rows
-      // ---- 2: weights
-      const bool test = x0 + cnt > W1;                      // (entries beyond the array carry no marks)
-      float s[SEC / NT];
+      for (int i = 0; i < EN; ++i) {
+        sm.idx[warp][t & 1][i * 32 + lane] = row_n[i];
+        tok_o[i] = entry(t, i) < r_end ? tok_n[i] : -1;
+        if (!KV || r_end > W1) sc_n[i] = tok_o[i] >= 0 ? __ldg(sc + tok_o[i]) : 0.f;
+      }
+      __syncwarp();
+      if ((t + 1) * NB < nbat) load(t + 1);
+    };
+    auto weigh = [&](int t) {                               // the open stage's weights
+      if (KV) dots(p, sm, bh, t, nbat);
 #pragma unroll
-      for (int i = 0; i < SEC / NT; ++i) s[i] = tok[i] >= 0 ? __ldg(sc + tok[i]) : 0.f;
-#pragma unroll
-      for (int i = 0; i < SEC / NT; ++i) {
-        bool on = tok[i] >= 0 && i * NT + tid < cnt;
-        if (test && on && x0 + i * NT + tid >= W1)
-          on = !in_topk(sm.mt, p.vtab + (long long)bh * VATTN_BANDCAP, p.bitmap + (long long)bh * p.nwords, tok[i], s[i]);
-        const float w = on ? expf((KV ? sm.w[i * NT + tid] : s[i]) - m) : 0.f;
-        sm.w[i * NT + tid] = w;
+      for (int i = 0; i < EN; ++i) {
+        bool on = tok_o[i] >= 0;
+        const int x = entry(t, i);
+        if (on && x >= W1)                                  // (entries beyond the array carry no marks)
+          on = !in_topk(sm.mt, p.vtab + (long long)bh * VATTN_BANDCAP, p.bitmap + (long long)bh * p.nwords, tok_o[i], sc_n[i]);
+        const float w = on ? expf((KV ? sm.w[warp][t & 1][i * 32 + lane] : sc_n[i]) - m) : 0.f;
+        sm.w[warp][t & 1][i * 32 + lane] = w;
         dd += w;
       }
-      __syncthreads();
-      // ---- 3: rows
+      __syncwarp();
+    };
+    auto issue = [&](int k, int slot_) {                    // batch k into a slot of the ring
+      if (k < nbat) {
+        const int4 id = *reinterpret_cast<const int4*>(&sm.idx[warp][(k / NB) & 1][(k % NB) * WB + rsub * UN]);
+        uint4 (&dst)[UN][32] = sm.warp[warp].ring[slot_];
+        cp_async16(&dst[0][lane], row_at<SPLIT>(p, vb, id.x));
+        cp_async16(&dst[1][lane], row_at<SPLIT>(p, vb, id.y));
+        cp_async16(&dst[2][lane], row_at<SPLIT>(p, vb, id.z));
+        cp_async16(&dst[3][lane], row_at<SPLIT>(p, vb, id.w));
+      }
+      cp_async_commit();
+    };
+    if (nbat > 0) {
+      load(0);
+      open(0);
+#pragma unroll
+      for (int k = 0; k < S; ++k) issue(k, k);
       int slot_ = 0;
 #pragma unroll 1
       for (int k = 0; k < nbat; ++k) {
-        const int at = k * CB + mine;
-        const float4 w4 = *reinterpret_cast<const float4*>(sm.w + at);
+        if (k % NB == 0) weigh(k / NB);
+        const float4 w4 = *reinterpret_cast<const float4*>(&sm.w[warp][(k / NB) & 1][(k % NB) * WB + rsub * UN]);
         const float w[UN] = {w4.x, w4.y, w4.z, w4.w};
         cp_async_wait<S - 1>();
         uint4 raw[UN];
 #pragma unroll
-        for (int u = 0; u < UN; ++u) raw[u] = sm.ring[warp][slot_][u][lane];
-        if ((k + 1) * CB > cnt) {                           // (uniform) padding must not count whatever its row holds
+        for (int u = 0; u < UN; ++u) raw[u] = sm.warp[warp].ring[slot_][u][lane];
+        if (k == nbat - 1) {                                // (uniform) padding must not count whatever its row holds
+          const int at = r_begin + k * CB + warp * WB + rsub * UN;
 #pragma unroll
-          for (int u = 0; u < UN; ++u) if (at + u >= cnt) raw[u] = make_uint4(0u, 0u, 0u, 0u);
+          for (int u = 0; u < UN; ++u) if (at + u >= r_end) raw[u] = make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
@@ -196,11 +193,12 @@ struct Gather {
 #pragma unroll
           for (int e = 0; e < EPL; ++e) acc[e] = fmaf(w[u], v[e], acc[e]);
         }
+        if ((k + S) % NB == 0 && k + S < nbat) open((k + S) / NB);
         issue(k + S, slot_);                                // (into the slot that has just been read)
         slot_ = slot_ == S - 1 ? 0 : slot_ + 1;
       }
+      cp_async_wait<0>();
     }
-    cp_async_wait<0>();
 #pragma unroll
     for (int mask = LPR; mask < 32; mask <<= 1) {
 #pragma unroll
@@ -208,17 +206,18 @@ struct Gather {
     }
 #pragma unroll
     for (int mask = 16; mask >= 1; mask >>= 1) dd += __shfl_xor_sync(FULL, dd, mask);
+    __syncwarp();                                           // (the warp's sums lie over its rows)
     if (rsub == 0) {
 #pragma unroll
-      for (int e = 0; e < EPL; ++e) sm.part[warp][j * EPL + e] = acc[e];
-      if (j == 0) sm.part[warp][D] = dd;
+      for (int e = 0; e < EPL; ++e) sm.warp[warp].part[j * EPL + e] = acc[e];
+      if (j == 0) sm.warp[warp].part[D] = dd;
     }
     __syncthreads();
     float* gpart = p.gat_part + ((long long)bh * p.gat_slots + slot) * NE;
     for (int e = tid; e < NE; e += NT) {
       float s = 0.f;
 #pragma unroll
-      for (int w = 0; w < NWARP; ++w) s += sm.part[w][e];
+      for (int w = 0; w < NWARP; ++w) s += sm.warp[w].part[e];
       gpart[e] = s;
     }
     // (the barrier orders every thread's writes before thread 0's fence, which is cumulative; likewise on the way in)
@@ -270,25 +269,26 @@ struct Gather {
       if (e < D) out[e] = Elem<T>::from_float((float)((det_e[it] + f * (double)num_s[it]) / den));
     }
   }
-  // K+V variant: scale <q, K[row]> of the section's rows to sm.w (what a selector that leaves no scores for the whole
-  // context behind would need), from rows in registers; all threads
-  static __device__ __forceinline__ void dots(const Prob& p, Sm& sm, int bh, int nbat, int mine) {
-    const int lane = threadIdx.x & 31, j = lane % LPR;
+  // K+V variant: scale <q, K[row]> of a stage's rows to sm.w (what a selector that leaves no scores for the whole
+  // context behind would need), from rows in registers; one warp
+  static __device__ __forceinline__ void dots(const Prob& p, Sm& sm, int bh, int t, int nbat) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane % LPR, rsub = lane / LPR;
     const int h = bh % p.Hq, b = bh / p.Hq, g = h / p.G;
     const char* kb = head_rows<T>(p, p.kc, g) + j * 16;
     float qf[EPL];
     Elem<T>::load(reinterpret_cast<const T*>(p.q) + q_row(p, b, h) + j * EPL, qf);
     uint4 r[UN];
     auto load = [&](int k) {
-      const int4 id = *reinterpret_cast<const int4*>(sm.idx + k * CB + mine);
+      const int4 id = *reinterpret_cast<const int4*>(&sm.idx[warp][t & 1][k * WB + rsub * UN]);
       r[0] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.x)));
       r[1] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.y)));
       r[2] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.z)));
       r[3] = __ldcs(reinterpret_cast<const uint4*>(row_at<SPLIT>(p, kb, id.w)));
     };
+    const int batches = min(NB, nbat - t * NB);
     load(0);
 #pragma unroll 1
-    for (int k = 0; k < nbat; ++k) {
+    for (int k = 0; k < batches; ++k) {
       float d[UN];
 #pragma unroll
       for (int u = 0; u < UN; ++u) {
@@ -298,7 +298,7 @@ struct Gather {
 #pragma unroll
         for (int e = 0; e < EPL; ++e) d[u] = fmaf(qf[e], x[e], d[u]);
       }
-      if (k + 1 < nbat) load(k + 1);
+      if (k + 1 < batches) load(k + 1);
       // a butterfly that hands rows over while it adds: lane j ends with the product of row own
       const bool a = (j & (LPR / 2)) != 0, c = (j & (LPR / 4)) != 0;
       const float y0 = (a ? d[2] : d[0]) + __shfl_xor_sync(FULL, a ? d[0] : d[2], LPR / 2);
@@ -306,9 +306,9 @@ struct Gather {
       float y = (c ? y1 : y0) + __shfl_xor_sync(FULL, c ? y0 : y1, LPR / 4);
 #pragma unroll
       for (int mask = LPR / 8; mask >= 1; mask >>= 1) y += __shfl_xor_sync(FULL, y, mask);
-      if (j % (LPR / 4) == 0) sm.w[k * CB + mine + (a ? 2 : 0) + (c ? 1 : 0)] = p.scale * y;
+      if (j % (LPR / 4) == 0) sm.w[warp][t & 1][k * WB + rsub * UN + (a ? 2 : 0) + (c ? 1 : 0)] = p.scale * y;
     }
-    __syncthreads();
+    __syncwarp();
   }
 };
 
