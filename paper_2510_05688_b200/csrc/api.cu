@@ -476,14 +476,17 @@ int vattn_decode(vattn_plan* plan, const void* q, const void* k_cache, const voi
   rc = prepare_stream(plan, p, st);
   if (rc != VATTN_OK) return rc;
   const bool was_clean = plan->clean;
+  // (the measurement aids look at the kernels one by one)
+  p.rows_cluster = plan->profiling || plan->stop_after != 0 ? 0 : rows_cluster(p);
   prof_mark(plan, 0, st);
   // score pass (walk tokens beside it) -> selection and sample lists (one CTA per head) -> deterministic and
   // base-sample rows (started per head by flags of the selection kernel), budget by the last CTA of a head -> final
   // sample, combination.  Every kernel is launched with programmatic dependent launch: its prologue
   // runs while its predecessor drains; the first one waits before it reads or writes anything.
   cudaError_t (*const launch[VATTN_NUM_KERNELS])(const Prob&, cudaStream_t) = {launch_score, launch_walk, launch_select,
-                                                                              launch_stats, launch_gather};
-  for (int i = 0; i < VATTN_NUM_KERNELS; ++i) {
+                                                                              p.rows_cluster ? launch_rows : launch_stats, launch_gather};
+  const int kernels = p.rows_cluster ? VATTN_NUM_KERNELS - 1 : VATTN_NUM_KERNELS;
+  for (int i = 0; i < kernels; ++i) {
     if (launch[i](p, st) != cudaSuccess) return cut_short(plan, p, st, was_clean, VATTN_ERR_CUDA);
     plan->last_launches++;
     prof_mark(plan, i + 1, st);

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2510_05688_b200 import synth
-from helpers import out_values, run_gpu, run_oracle
+from helpers import assert_parity, out_values, run_gpu, run_oracle
 from test_gpu_parity import check, small
 
 pytestmark = pytest.mark.gpu
@@ -206,3 +206,33 @@ def test_paths_tell_where_the_bound_came_from():
     assert (dbg["paths"][:148] & 17 == 1).all() and (dbg["paths"][148] & 17 == 16).all()
     _, dbg, plan = run_gpu(small("bf16", [700, 70000], Hq=1, Hkv=1, d=64, k=100))
     assert (dbg["paths"] & 17 == 1).all()
+
+
+@pytest.mark.parametrize("dtype,B,Hq,Hkv,d,max_len", [
+    ("fp32", 1, 1, 1, 64, None), ("bf16", 1, 16, 2, 128, None), ("bf16", 2, 8, 8, 64, None), ("bf16", 17, 1, 1, 128, None),
+    ("fp32", 4, 8, 2, 128, 16384), ("fp32", 4, 8, 2, 64, 16400), ("fp32", 11, 3, 3, 64, None)])
+def test_rows_of_a_head_in_one_kernel_and_in_two(dtype, B, Hq, Hkv, d, max_len):
+    # 16 | 17 heads, 32 | 33 fp32 heads and 16,384 | 16,385 tokens: one kernel for statistics, budget and gather, or two (which
+    # the measurement aids always take).  Empty and one-token rows, no middle range, budgets up to the whole residual, listed
+    # samples, nested samples, fewer rows than CTAs.
+    from paper_2510_05688_b200 import binding as vb
+    lens = ([1501, 0, 1, 13] + [(97 * i) % 900 + 40 for i in range(B)])[:B]
+    case = small(dtype, lens, Hq=Hq, Hkv=Hkv, d=d, k=37, params=dict(base_rate=0.03))
+    fused = B * Hq <= (32 if dtype == "fp32" and (max_len or 0) <= 16384 else 16)
+    width = 16 * case.max_blocks_per_seq if max_len is None else max_len
+    if width > 16 * case.max_blocks_per_seq:
+        table = np.zeros((B, (width + 15) // 16), case.block_table.dtype)
+        table[:, :case.max_blocks_per_seq] = case.block_table
+        case.block_table = table
+    for over in ({}, dict(force_budget=1), dict(force_budget=700), dict(force_budget=1 << 20), dict(nested_base=1), dict(base_rate=0.9)):
+        out_ref, det = run_oracle(case, **over)
+        for two in (False, True):
+            plan = vb.plan_for_case(case, max_seq_len=width)
+            plan.set_profiling(two)
+            out, dbg, _ = run_gpu(case, plan=plan, **over)
+            one = fused and not two and 4 + 8 + 37 + over.get("base_rate", 0.03) * width <= 4096
+            assert plan.last_launch_count() == (4 if one else 5)
+            assert_parity(case, out, dbg, det, out_ref)
+            assert plan.last_status() == 0
+            plain, _, _ = run_gpu(case, debug=False, plan=plan, **over)
+            assert np.array_equal(plain, out)
