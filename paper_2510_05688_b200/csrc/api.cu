@@ -125,9 +125,9 @@ void derive(vattn_plan* pl) {
   pl->off_topk = take(2 * BH * pl->npad * sizeof(int));     // tokens, row indices
   pl->off_selcnt = take(2 * BH * (pl->npad / 16 + 32) * sizeof(int));
   pl->off_walk = take(4 * BH * pl->npad * sizeof(int));     // first walk positions of both walks: tokens, row indices
-  pl->off_holes = take(2 * BH * VATTN_BANDCAP * sizeof(int));
+  pl->off_holes = take(BH * VATTN_BANDCAP * sizeof(int));
   pl->off_wkeys = take(BH * 8 * sizeof(unsigned));
-  pl->off_dyn = take(3 * BH * pl->npad * sizeof(int));      // tokens, row indices; 64-bit keys of the near-tie overflow path
+  pl->off_dyn = take(3 * BH * pl->npad * sizeof(int));      // tokens, row indices (64-bit keys of the near-tie overflow path); far positions
   pl->off_meta = take(BH * sizeof(HeadMeta));
   pl->off_stat = take(BH * 2 * VATTN_STAT_MAXS * (D + 3) * sizeof(double));
   pl->off_piv = take(BH * (D + 1) * sizeof(double));

@@ -811,7 +811,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
   //      kernel, which start after this kernel has completed)
   if (n_s > 0) {
     int* cnts = sm.misc;                               // members inside the walk array, beyond it
-    int* hp1 = p.hole_pos + (long long)bh * 2 * VATTN_BANDCAP;     // positions inside the walk array; + BANDCAP: beyond it
+    int* hp1 = p.hole_pos + (long long)bh * VATTN_BANDCAP;         // positions inside the walk array
+    int* hp2 = p.dyn_idx + ((long long)bh * 3 + 2) * p.npad;       // ... and beyond it
     const Walk wk1 = make_walk(sm.rkeys + 8, mlen);
     if (tid < 2) cnts[tid] = 0;
     __syncthreads();
@@ -822,18 +823,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select(const __grid_constant_
         const int i1 = atomicAdd(&cnts[0], 1);
         if (i1 < VATTN_BANDCAP) hp1[i1] = x1;
       } else {                                         // (budgets that reach beyond the array need these)
-        const int i2 = atomicAdd(&cnts[1], 1);
-        if (i2 < VATTN_BANDCAP) hp1[VATTN_BANDCAP + i2] = x1;
+        hp2[atomicAdd(&cnts[1], 1)] = x1;
       }
     }
     __syncthreads();
     if (tid == 0) {
       const int holes1 = cnts[0], holes2 = cnts[1];
-      // every member's position is known: any budget can be served as "the non-members among the first J
-      // positions" (entries beyond the array are computed by the gather kernel); else only budgets inside the array
+      // every member's position is known: any budget can be served as "the non-members among the first J positions"
+      // (entries beyond the array are computed by the gather).  More marks in the array than the list holds: none can.
       HeadMeta* gm = p.meta + bh;
-      gm->holes1 = min(holes1, VATTN_BANDCAP); gm->holes2 = min(holes2, VATTN_BANDCAP);
-      if (holes1 <= VATTN_BANDCAP) { gm->dyn_J = W1; gm->dyn_listed = holes2 <= VATTN_BANDCAP ? n_s : W1 - holes1; }
+      gm->holes1 = min(holes1, VATTN_BANDCAP); gm->holes2 = holes2;
+      if (holes1 <= VATTN_BANDCAP) { gm->dyn_J = W1; gm->dyn_listed = n_s; }
     }
   }
   // ---- introspection: I_t ascending (a bitmap of the tokens in shared memory), I_bs in walk order

@@ -153,6 +153,39 @@ __device__ __noinline__ void list_sample(const Prob& p, int b, int h, int bh, in
   }
 }
 
+// The least J with bfin unmarked positions below it, for budgets beyond the walk array and more members of I_t out there than
+// the threads hold in registers (see head_budget): every step reads the positions again.
+__device__ __noinline__ int far_prefix(int bfin, const int* near, int n_near, const int* far, int n_far, int most, int* cnt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int turn = 0;
+  auto marked_below = [&](int Jq) {                        // (uniform over the CTA)
+    int c = 0;
+    for (int i = threadIdx.x; i < n_near; i += NT) c += __ldcg(near + i) < Jq;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n_far; i += NT) c += __ldcg(far + i) < Jq;
+    c = __reduce_add_sync(FULLMASK, c);
+    if (lane == 0) cnt[turn * NWARP + warp] = c;
+    __syncthreads();
+    int t = 0;
+#pragma unroll
+    for (int w = 0; w < NWARP; ++w) t += cnt[turn * NWARP + w];
+    turn ^= 1;
+    return t;
+  };
+  int J = bfin;
+  for (int it = 0; it < 8; ++it) {
+    const int c = marked_below(J);
+    if (bfin + c == J) return J;
+    J = bfin + c;
+  }
+  int hi = most, lo = min(J, hi);
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (mid - marked_below(mid) >= bfin) hi = mid; else lo = mid + 1;
+  }
+  return lo;
+}
+
 // Budget of head bh from the partials of its S0 + S1 CTAs, by the last of them.  It stands between the rows and the
 // gather of every head, so it is a short chain: everything it reads is requested at once (one round trip), thread e
 // adds element e of both kinds in split order, warp k the k-th scalar sum, one barrier, and every warp evaluates the
@@ -171,7 +204,7 @@ __device__ __forceinline__ HeadBudget head_budget(const Prob& p, int bh, int S0,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const HeadMeta mt = ld_meta(p.meta + bh);
   // the marked positions of the final sample's walk array, eight per thread (what lies behind the last one is ignored)
-  const int* hd = p.hole_pos + (long long)bh * 2 * VATTN_BANDCAP;
+  const int* hd = p.hole_pos + (long long)bh * VATTN_BANDCAP;
   static_assert(VATTN_BANDCAP == 8 * NT, "eight positions per thread");
   int hp[8];
 #pragma unroll
@@ -266,13 +299,14 @@ __device__ __forceinline__ HeadBudget head_budget(const Prob& p, int bh, int S0,
   int J = bfin, start = 0;
   if (!listed && bfin >= n_s) J = mt.l_start - mt.s0;      // the whole residual: every middle token, in token order
   else if (!listed) {
-    const int nholes = min(max(mt.holes1, 0), VATTN_BANDCAP), nholes2 = min(max(mt.holes2, 0), VATTN_BANDCAP);
+    const int nholes = min(max(mt.holes1, 0), VATTN_BANDCAP), nholes2 = min(max(mt.holes2, 0), p.npad);
+    const int* hd2 = p.dyn_idx + ((long long)bh * 3 + 2) * p.npad;
     const bool far = bfin > mt.dyn_J - nholes;             // reaches beyond the walk array: the members there count too
     int hf[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       if (i * NT + tid >= nholes) hp[i] = 0x7FFFFFFF;
-      hf[i] = far && i * NT + tid < nholes2 ? __ldcg(hd + VATTN_BANDCAP + i * NT + tid) : 0x7FFFFFFF;
+      hf[i] = far && i * NT + tid < nholes2 ? __ldcg(hd2 + i * NT + tid) : 0x7FFFFFFF;
     }
     int* cnt = reinterpret_cast<int*>(scal + 16);          // [2][NWARP], taken in turn
     int turn = 0;
@@ -289,19 +323,22 @@ __device__ __forceinline__ HeadBudget head_budget(const Prob& p, int bh, int S0,
       turn ^= 1;
       return t;
     };
-    bool conv = false;
-    for (int it = 0; it < 8; ++it) {
-      const int c = marked_below(J);
-      if (bfin + c == J) { conv = true; break; }
-      J = bfin + c;
-    }
-    if (!conv) {
-      int hi_ = far ? mt.l_start - mt.s0 : mt.dyn_J, lo_ = min(J, hi_);
-      while (lo_ < hi_) {
-        const int mid = (lo_ + hi_) >> 1;
-        if (mid - marked_below(mid) >= bfin) hi_ = mid; else lo_ = mid + 1;
+    if (far && nholes2 > 8 * NT) J = far_prefix(bfin, hd, nholes, hd2, nholes2, mt.l_start - mt.s0, cnt);
+    else {
+      bool conv = false;
+      for (int it = 0; it < 8; ++it) {
+        const int c = marked_below(J);
+        if (bfin + c == J) { conv = true; break; }
+        J = bfin + c;
       }
-      J = lo_;
+      if (!conv) {
+        int hi_ = far ? mt.l_start - mt.s0 : mt.dyn_J, lo_ = min(J, hi_);
+        while (lo_ < hi_) {
+          const int mid = (lo_ + hi_) >> 1;
+          if (mid - marked_below(mid) >= bfin) hi_ = mid; else lo_ = mid + 1;
+        }
+        J = lo_;
+      }
     }
     // nested samples: the base sample's rows are the first b0 rows of I_dyn and their sums are known here (in fp64, from
     // rescored weights): they are folded into the deterministic sums (scaled like the sample), and the gather kernel

@@ -34,7 +34,7 @@ struct HeadMeta {
   int dyn_J;        //   sample's walk" (dyn_J positions are in the walk array, members marked), larger ones from a list
   int path;         // code path of the selection (vattn_debug.paths)
   int base_J;       // the base sample = the unmarked entries among the first base_J of its walk array
-  int holes2;       // members of I_t at positions of the final sample's walk beyond its array (hole_pos + BANDCAP)
+  int holes2;       // members of I_t at positions of the final sample's walk beyond its array (the third part of dyn_idx)
   int holes1;       // marked entries among the first dyn_J of the final sample's walk (their positions in hole_pos)
   int pad[3];
 };
@@ -106,10 +106,11 @@ struct Prob {
                           //   walk the tokens, then their row indices.  The selection kernel marks the members
                           //   of I_t (token = -1; the row index stays valid): a sample is the unmarked entries of a prefix
   unsigned* wkeys;        // [B,Hq,8] round keys of the final sample's walk (for the gather kernel's array extension)
-  int* hole_pos;          // [B,Hq,2,VATTN_BANDCAP] positions of the marked entries of the final sample's walk array, in
-                          //   no particular order; then the positions of the members of I_t beyond the array (counts: HeadMeta)
-  int* dyn_idx;           // [B,Hq,3,npad] I_dyn as a list (tokens, row indices) for budgets beyond the walk arrays
-                          //               (scratch of the near-tie overflow path while the selection runs)
+  int* hole_pos;          // [B,Hq,VATTN_BANDCAP] positions of the marked entries of the final sample's walk array, in
+                          //   no particular order (count: HeadMeta)
+  int* dyn_idx;           // [B,Hq,3,npad] I_dyn as a list (tokens, row indices) where the known positions do not serve the
+                          //               budget (scratch of the near-tie overflow path while the selection runs); the
+                          //               positions of the members of I_t beyond the final sample's walk array
   HeadMeta* meta;         // [B,Hq]
   double* stat_part;      // [B,Hq,2*16,D+3]  partials of the statistics kernel (deterministic-row CTAs, then base-row CTAs)
   double* stat_piv;       // [B,Hq,D+1] pivot row of the base-sample sums: w*V then w

@@ -236,3 +236,16 @@ def test_rows_of_a_head_in_one_kernel_and_in_two(dtype, B, Hq, Hkv, d, max_len):
             assert plan.last_status() == 0
             plain, _, _ = run_gpu(case, debug=False, plan=plan, **over)
             assert np.array_equal(plain, out)
+
+
+@pytest.mark.parametrize("heads,k", [(2, 1500), (17, 1500), (2, 1110), (2, 1000)])
+def test_budgets_beyond_the_walk_array_with_many_members_there(heads, k):
+    # more members of I_t at walk positions beyond the array than a list of 1,024 holds: the budget counts them all
+    case = small("bf16", [9000], Hq=heads, Hkv=1, d=64, k=k, eps=0.1, delta=0.1, params=dict(base_rate=0.01))
+    out, dbg, det, plan = check(case)
+    b0 = det[(0, 0)]["b0"]
+    far = [r["b"] for r in det.values() if 8 * b0 < r["b"] < r["n_s"]]
+    assert far                                          # (beyond the array, short of the whole residual)
+    assert plan.last_status() == 0
+    for mode in (1, 2):
+        check(case, mode=mode)
