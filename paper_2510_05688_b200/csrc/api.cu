@@ -210,6 +210,7 @@ int fill_prob(const vattn_plan* pl, Prob& p, const void* q, const void* kc, cons
   // which leave some of the SMs' room free (256 there: 67.8 instead of 63.3 us per step at 96 heads x 8,192 tokens), 256
   // beyond (128 there: 74 instead of 69 us at 256 x 2,049; 512: 65 instead of 63)
   p.stat_rows = BH > 128 ? 256 : (5 * device_sm_count()) / (int)BH < 8 ? 64 : 48;
+  p.stat_by_row = pl->stat_splits > 1;
   p.dbg = pl->dbg;
   return VATTN_OK;
 }

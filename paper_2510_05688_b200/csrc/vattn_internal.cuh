@@ -119,6 +119,7 @@ struct Prob {
   int gat_slots;          // partial slots (chunks) per head: 16; 32 for up to 32 heads, 64 to 128 for up to 16
   int stat_splits, stat_splits_base;   // statistics CTAs per head, at most: deterministic rows, base-sample rows
   int stat_rows;          // rows that warrant a statistics CTA
+  int stat_by_row;        // dispatch order of its CTAs: both kinds of a batch row together
   int rows_cluster;       // CTAs per head of the fused rows kernel (0: the statistics and the gather run as two kernels)
   float* dense_part;      // [B,Hq,dense_splits,dense_rec(D)]
   int dense_splits;
