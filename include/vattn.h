@@ -113,7 +113,7 @@ typedef struct {
                                      select ran (VATTN_STATUS_BAND_OVERFLOW) */
   unsigned long long *kernel_ticks; /* [VATTN_NUM_TICKS][2] device-side time stamps in ns (%globaltimer): rows 1-5
                                      the score kernel, the walk kernel, the selection kernel, the statistics kernel and
-                                     the gather kernel, row 0 unused ([k][0] = earliest CTA start,
+                                     the gather kernel (of few heads: the two parts of one kernel), row 0 unused ([k][0] = earliest CTA start,
                                      [k][1] = latest end); row 6 the top-k selection proper (first CTA past its
                                      dependency wait .. last CTA with I_t complete); row 7 the budgets (first head
                                      whose statistics are complete .. last head that knows its budget).
@@ -250,7 +250,8 @@ int vattn_set_stop_after(vattn_plan* plan, int kernels);
 /* Optional per-kernel timing of vattn_decode, for measurement harnesses.  While enabled, every call
  * records CUDA events on `stream` around each of its VATTN_NUM_KERNELS kernels (score pass; walk tokens;
  * selection and sample lists; deterministic and base-sample rows with the budget; final sample and combination),
- * for up to 256 calls between two reads.  The events keep a kernel's prologue from running beside its predecessor, so the times add up to
+ * for up to 256 calls between two reads.  (For few heads the step otherwise runs its last two kernels as one; calls that
+ * are profiled or stopped early run them apart.)  The events keep a kernel's prologue from running beside its predecessor, so the times add up to
  * more than an unprofiled step takes.  vattn_read_profile waits for the last recorded call, writes the
  * summed elapsed milliseconds per kernel to ms_sum[VATTN_NUM_KERNELS] (host) and the number of calls to
  * *calls (host), and starts a new window.  Events add a little latency: do not enable in production. */
