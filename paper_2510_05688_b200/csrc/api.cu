@@ -90,7 +90,7 @@ void derive(vattn_plan* pl) {
   const int groups = s.batch * s.num_kv_heads * GC;
   const int sp = (8 * device_sm_count() + groups - 1) / groups;
   pl->dense_splits = sp < 1 ? 1 : (sp > 128 ? 128 : sp);
-  // statistics kernel (128-thread CTAs, 5 per SM): one wave for both kinds of CTA, half each, on the SMs that the selection
+  // statistics kernel (128-thread CTAs, 4 or 5 per SM): one wave for both kinds of CTA, half each, on the SMs that the selection
   // leaves free (with few heads it holds one SM per head until after the rows have been published: CTAs beyond that
   // started 4 us late; 151.9 -> 148.5 us per step at 32 heads of 131,071 tokens, others within 1 %).  From 70 heads on
   // four CTAs per kind and head overfill that wave and the kernel is throughput-bound: four all the same, so that the first
@@ -100,7 +100,7 @@ void derive(vattn_plan* pl) {
   // Both lines at three quarters of these counts: 79.9 instead of 75.2 us at 288 x 2,049 and 220 instead of 210 at 288 x
   // 4,096 to 32,768, 154.4 instead of 151.7 at 144 x 32,768; 175.5 instead of 177.3 at 184.
   {
-    const int sms = device_sm_count(), wave = 5 * (sms - (heads < sms / 4 ? heads : sms / 4)) / heads;
+    const int sms = device_sm_count(), wave = stat_ctas_per_sm(heads) * (sms - (heads < sms / 4 ? heads : sms / 4)) / heads;
     if (wave < 8) {
       const int full = 5 * sms / heads;
       pl->stat_splits = pl->stat_splits_base = full < 2 ? 1 : full < 4 ? 2 : 4;
@@ -282,6 +282,12 @@ int cut_short(vattn_plan* pl, const Prob& p, cudaStream_t st, bool was_clean, in
 }
 
 }  // namespace
+
+// CTAs per SM of the statistics kernel.  Five (96 registers) where its CTAs outnumber the places.  Where all of them fit, four
+// with 128 registers, whose chains of fixed latencies the compiler can interleave more: 62.1 -> 61.4 us per step at 32 heads x
+// 32,768 tokens, 147.3 -> 146.3 at 131,071, 62.3 -> 61.6 at 64 x 16,384, but 199.2 -> 201.4 at 256 x 32,768 and 108.6 -> 109.6 at
+// 128 x 32,768.  (Six with 80: 64.7, 202.9 and 111.6.)
+int stat_ctas_per_sm(int heads) { return heads <= device_sm_count() / 2 ? 4 : 5; }
 
 int device_sm_count() {
   static int cached[VATTN_MAXDEV];

@@ -26,8 +26,9 @@
 
 namespace {
 
-template <typename T, int D, bool SPLIT>
-__global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p) {
+// CTAS: CTAs per SM (see stat_ctas_per_sm)
+template <typename T, int D, bool SPLIT, int CTAS>
+__global__ void __launch_bounds__(NT, CTAS) k_stats(const __grid_constant__ Prob p) {
   constexpr int NE = D + 3;               // det CTA: N_f[D], D_f;  base CTA: Sr[D], Sw, Sww, Srr
   using R = StatRows<T, D, SPLIT>;
   __shared__ typename R::Sm sm;
@@ -156,17 +157,18 @@ __global__ void __launch_bounds__(NT, 5) k_stats(const __grid_constant__ Prob p)
 
 }  // namespace
 
-template <typename T, int D, bool SPLIT>
+template <typename T, int D, bool SPLIT, int CTAS>
 static cudaError_t launch_stats_n(const Prob& p, cudaStream_t s) {
   static size_t have[VATTN_MAXDEV];
-  cudaError_t e = optin_smem(k_stats<T, D, SPLIT>, 0, have, true);
+  cudaError_t e = optin_smem(k_stats<T, D, SPLIT, CTAS>, 0, have, true);
   if (e != cudaSuccess) return e;
   const dim3 grid(p.stat_splits > p.stat_splits_base ? p.stat_splits : p.stat_splits_base, p.Hq, 2 * p.B);
-  return launch_pdl(k_stats<T, D, SPLIT>, grid, dim3(NT), 0, s, p);
+  return launch_pdl(k_stats<T, D, SPLIT, CTAS>, grid, dim3(NT), 0, s, p);
 }
 template <typename T, int D>
 static cudaError_t launch_stats_t(const Prob& p, cudaStream_t s) {
-  return p.row_unit == 0u ? launch_stats_n<T, D, true>(p, s) : launch_stats_n<T, D, false>(p, s);
+  if (p.row_unit == 0u) return launch_stats_n<T, D, true, 5>(p, s);      // (rare: one form)
+  return stat_ctas_per_sm(p.B * p.Hq) == 4 ? launch_stats_n<T, D, false, 4>(p, s) : launch_stats_n<T, D, false, 5>(p, s);
 }
 
 cudaError_t launch_stats(const Prob& p, cudaStream_t s) {

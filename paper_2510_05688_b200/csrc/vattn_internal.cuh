@@ -568,6 +568,7 @@ cudaError_t launch_score(const Prob& p, cudaStream_t s);
 cudaError_t launch_walk(const Prob& p, cudaStream_t s);
 int select_threads(const Prob& p);
 cudaError_t launch_select(const Prob& p, cudaStream_t s);
+int stat_ctas_per_sm(int heads);
 cudaError_t launch_stats(const Prob& p, cudaStream_t s);
 cudaError_t launch_gather(const Prob& p, cudaStream_t s);
 int rows_cluster(const Prob& p);                         // (see Prob::rows_cluster)
