@@ -30,8 +30,10 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(NT, 5) k_rows(const __grid_constant__ Prob p, int C) {
+// CTAS: CTAs per SM.  Four (128 registers) up to 16 heads: 24.6 -> 24.2 us per step at one fp32 head of 1,024 tokens, 35.8 -> 34.9
+// at 16 x 4,096; 32 clusters need five (41.7 against 50.6 at 32 fp32 heads).
+template <typename T, int D, int CTAS>
+__global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob p, int C) {
   using R = StatRows<T, D, false>;
   using G = Gather<T, D, false, false>;
   constexpr int NE = D + 3, NG = D + 1;
@@ -161,16 +163,16 @@ __global__ void __launch_bounds__(NT, 5) k_rows(const __grid_constant__ Prob p, 
   }
 }
 
-template <typename T, int D>
-cudaError_t launch_rows_t(const Prob& p, int C, cudaStream_t s, int* fit) {
+template <typename T, int D, int CTAS>
+cudaError_t launch_rows_n(const Prob& p, int C, cudaStream_t s, int* fit) {
   static size_t have[VATTN_MAXDEV];
-  cudaError_t e = optin_smem(k_rows<T, D>, 0, have, true);
+  cudaError_t e = optin_smem(k_rows<T, D, CTAS>, 0, have, true);
   if (e != cudaSuccess) return e;
   static int wide[VATTN_MAXDEV];                   // clusters beyond the portable size are allowed
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if (C > 8 && !__atomic_load_n(&wide[dev], __ATOMIC_ACQUIRE)) {
-    if ((e = cudaFuncSetAttribute(k_rows<T, D>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_rows<T, D, CTAS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     __atomic_store_n(&wide[dev], 1, __ATOMIC_RELEASE);
   }
   cudaLaunchConfig_t cfg = {};
@@ -183,10 +185,16 @@ cudaError_t launch_rows_t(const Prob& p, int C, cudaStream_t s, int* fit) {
   cfg.attrs = attr;
   if (fit) {
     cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(fit, k_rows<T, D>, &cfg);
+    return cudaOccupancyMaxActiveClusters(fit, k_rows<T, D, CTAS>, &cfg);
   }
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k_rows<T, D>, p, C);
+  return cudaLaunchKernelEx(&cfg, k_rows<T, D, CTAS>, p, C);
+}
+template <typename T, int D>
+cudaError_t launch_rows_t(const Prob& p, int C, cudaStream_t s, int* fit) {
+  if constexpr (sizeof(T) == 4)
+    if (p.B * p.Hq > 16) return launch_rows_n<T, D, 5>(p, C, s, fit);
+  return launch_rows_n<T, D, 4>(p, C, s, fit);
 }
 cudaError_t launch_rows_any(const Prob& p, int C, cudaStream_t s, int* fit) {
   if (p.dtype == VATTN_DTYPE_BF16) return p.D == 128 ? launch_rows_t<bf16_t, 128>(p, C, s, fit) : launch_rows_t<bf16_t, 64>(p, C, s, fit);
@@ -212,10 +220,10 @@ int rows_cluster(const Prob& p) {
   const double msl = (double)p.max_seq_len, kmax = p.topk_frac > 0.f ? (double)p.topk_frac * msl : (double)p.k;
   if ((double)p.sink + (double)p.window + kmax + (double)p.base_rate * msl > 256.0 * C) return 0;
   // (a device that cannot hold such a cluster takes the two kernels)
-  static signed char ok[VATTN_MAXDEV][2][2];
+  static signed char ok[VATTN_MAXDEV][2][2][2];
   int dev = 0, fit = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= VATTN_MAXDEV) { cudaGetLastError(); return 0; }
-  signed char* known = &ok[dev][p.dtype == VATTN_DTYPE_BF16][p.D == 128];
+  signed char* known = &ok[dev][p.dtype == VATTN_DTYPE_BF16][p.D == 128][heads <= 16];
   signed char k = __atomic_load_n(known, __ATOMIC_ACQUIRE);
   if (k == 0) {
     k = launch_rows_any(p, C, nullptr, &fit) == cudaSuccess && fit >= 1 ? 1 : -1;
