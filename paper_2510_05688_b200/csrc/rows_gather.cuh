@@ -18,6 +18,7 @@
 // row, issued about 250 instructions per eight rows and reached half the bandwidth.)
 #pragma once
 #include "vattn_internal.cuh"
+#include <stddef.h>
 
 namespace {
 
@@ -38,8 +39,8 @@ struct Gather {
     __device__ WarpMem() {}
   };
   struct Stages {
-    int idx[NWARP][2][32 * EN];                             // row indices of two stages
-    float w[NWARP][2][32 * EN];                             // weights
+    alignas(16) int idx[NWARP][2][32 * EN];                 // row indices of two stages
+    alignas(16) float w[NWARP][2][32 * EN];                 // weights
     unsigned keys[8];
     HeadMeta mt;
     GMeta meta;
@@ -55,6 +56,8 @@ struct Gather {
   struct Sm : Rings, Stages {
     __device__ Sm() {}
   };
+  // (a user of the stages declares them alone, and a lane reads four row indices or weights as one 16-byte word)
+  static_assert(alignof(Stages) >= 16 && offsetof(Stages, idx) % 16 == 0 && offsetof(Stages, w) % 16 == 0, "four indices or weights per read");
   static __device__ __forceinline__ void unpack(const uint4& r, float (&v)[EPL]) {
     if (EPL == 8) {
       v[0] = __uint_as_float(r.x << 16); v[1] = __uint_as_float(r.x & 0xFFFF0000u);
