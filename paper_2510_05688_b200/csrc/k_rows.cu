@@ -31,7 +31,7 @@ __device__ __forceinline__ void cluster_sync() {
 }
 
 // CTAS: CTAs per SM.  Four (128 registers) up to 16 heads: 24.6 -> 24.2 us per step at one fp32 head of 1,024 tokens, 35.8 -> 34.9
-// at 16 x 4,096; 32 clusters need five (41.7 against 50.6 at 32 fp32 heads).
+// at 16 x 4,096; 32 clusters need five (41.7 against 50.6 at 32 fp32 heads of 64 elements).
 template <typename T, int D, int CTAS>
 __global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob p, int C) {
   using R = StatRows<T, D, false>;
@@ -192,7 +192,7 @@ cudaError_t launch_rows_n(const Prob& p, int C, cudaStream_t s, int* fit) {
 }
 template <typename T, int D>
 cudaError_t launch_rows_t(const Prob& p, int C, cudaStream_t s, int* fit) {
-  if constexpr (sizeof(T) == 4)
+  if constexpr (sizeof(T) == 4 && D == 64)
     if (p.B * p.Hq > 16) return launch_rows_n<T, D, 5>(p, C, s, fit);
   return launch_rows_n<T, D, 4>(p, C, s, fit);
 }
@@ -206,19 +206,32 @@ cudaError_t launch_rows_any(const Prob& p, int C, cudaStream_t s, int* fit) {
 cudaError_t launch_rows(const Prob& p, cudaStream_t s) { return launch_rows_any(p, p.rows_cluster, s, nullptr); }
 
 // CTAs per head of the fused kernel; 0: the statistics and the gather run as two kernels.  Up to 16 heads a cluster of 16
-// per head leaves most SMs to themselves: 28.3 -> 23.7 us per step at one fp32 head of 1,024 tokens, 45.6 -> 38.0 at 4 fp32
-// heads x 12,795, 45.0 -> 40.7 at 8 bf16 heads x 16,384, 48.7 -> 47.4 at 16 x 32,768.  Beyond that the clusters, which need
-// 16 places in one GPC, load the SMs unevenly and a head waits for its slowest CTA: 62.5 -> 64.9 at 32 x 32,768, 43.8 -> 45.5
-// at 32 x 8,192, 106 -> 132 at 128 x 32,768 with 4 CTAs each.  fp32 has them up to 32 heads where the selection's CTAs
-// (512 threads then, see select_threads) leave room on their SMs: 42.7 -> 41.2 at 32 x 6,000 to 9,000, 45.8 -> 44.4 at 32 x
-// 16,000, but 78.9 -> 80.7 at 32 x 30,000.  More rows than 256 per CTA: two kernels, which have up to 32 CTAs per head for
-// the statistics (104.2 -> 106.8 at 8 heads x 100,001 tokens).
+// per head leaves most SMs to themselves: 28.3 -> 23.7 us per step at one fp32 head of 1,024 tokens, 33.9 -> 28.9 at one bf16
+// head that samples a fifth of 4,096, 41.2 -> 33.6 at a fifth of 12,800.  Beyond that the clusters, which need 16 places in one
+// GPC, load the SMs unevenly and a head waits for its slowest CTA: 62.5 -> 64.9 at 32 x 32,768, 43.8 -> 45.5 at 32 x 8,192.
+// fp32 rows of 64 elements have them up to 32 heads where the selection's CTAs (512 threads then, see select_threads) leave
+// room on their SMs: 33.0 -> 31.4 at 32 x 2,048, 30.6 -> 28.5 at 17, but at rows of 128 elements 35.9 -> 37.1 at 32 x 2,048
+// and 45.7 -> 48.6 at 24 x 9,001.
+// More deterministic and base rows than 256 per CTA: two kernels, which have up to 32 CTAs per head for the statistics (104.2 ->
+// 106.8 at 8 heads x 100,001 tokens).  The sampled rows count as well, as many as the call may take, for the budget is known on
+// the GPU only: 16 CTAs keep 384 KB of a head's rows in flight, where the two kernels spread them over up to 128 CTAs.  With
+// every residual token sampled, at rows of 256 bytes: one head 43.1 -> 41.8 at 12,800 tokens, 43.0 -> 43.3 at 16,384, 49.1 ->
+// 59.7 at 32,768; four heads 43.8 -> 45.5 at 16,384; eight 44.5 -> 44.4 at 10,000, 44.2 -> 47.7 at 16,384; 16 heads 40.0 -> 42.1
+// at 8,000, 64.8 -> 78.5 at 32,768; 32 fp32 heads 32.5 -> 31.0 at 2,048, 40.9 -> 41.2 at 6,000, 55.9 -> 58.1 at 16,000.  At 512
+// bytes one head 39.1 -> 37.7 at 8,000 and 39.6 -> 46.9 at 16,384; at 128 bytes 41.8 -> 41.0 at 16,384 and 44.0 -> 50.5 at
+// 32,768.  Hence at most 16,384 rows and 4 MB of a head and 16 MB of all heads.  (Kept beyond that for budgets that turn out
+// small it would save up to 5 us.  Both ways to leave only the large ones to more CTAs cost what they saved: a gather kernel
+// behind it 2 us, 46.7 -> 46.5 and 50.6 -> 53.2 at 8 and 16 heads x 32,768; clusters without a head of their own that wait for
+// the budgets 3 to 12 us.)
 int rows_cluster(const Prob& p) {
   if (p.row_unit == 0u || p.gather_kv) return 0;
   const int heads = p.B * p.Hq, C = VATTN_ROWS_CLUSTER;
-  if (heads > (p.dtype == VATTN_DTYPE_FP32 && p.max_seq_len <= 16384 ? 32 : 16)) return 0;
+  if (heads > (p.dtype == VATTN_DTYPE_FP32 && p.D == 64 && p.max_seq_len <= 16384 ? 32 : 16)) return 0;
   const double msl = (double)p.max_seq_len, kmax = p.topk_frac > 0.f ? (double)p.topk_frac * msl : (double)p.k;
   if ((double)p.sink + (double)p.window + kmax + (double)p.base_rate * msl > 256.0 * C) return 0;
+  const int sampled = p.force_budget >= 0 && p.force_budget < p.max_seq_len ? p.force_budget : p.max_seq_len;
+  const long long bytes = (long long)sampled * p.D * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4);
+  if (sampled > 16384 || bytes > 4ll << 20 || heads * bytes > 16ll << 20) return 0;
   // (a device that cannot hold such a cluster takes the two kernels)
   static signed char ok[VATTN_MAXDEV][2][2][2];
   int dev = 0, fit = 0;
