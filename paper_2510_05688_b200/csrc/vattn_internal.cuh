@@ -220,11 +220,14 @@ template <> struct Elem<bf16_t> {
   }
 };
 
-// physical page of logical page `lp` of batch row b (bounds-checked; a bad entry raises a status bit)
-__device__ __forceinline__ int page_of(const Prob& p, int b, int lp) {
-  int pg = p.bt[(long long)b * p.max_blocks + lp];
+__device__ __forceinline__ int table_entry(const Prob& p, int b, int lp) { return p.bt[(long long)b * p.max_blocks + lp]; }
+__device__ __forceinline__ int checked_page(const Prob& p, int pg) {
   if ((unsigned)pg >= (unsigned)p.num_blocks) { atomicOr(p.status, VATTN_STATUS_BAD_BLOCK); pg = 0; }
   return pg;
+}
+// physical page of logical page `lp` of batch row b (bounds-checked; a bad entry raises a status bit)
+__device__ __forceinline__ int page_of(const Prob& p, int b, int lp) {
+  return checked_page(p, table_entry(p, b, lp));
 }
 template <typename T>
 __device__ __forceinline__ const T* row_ptr(const Prob& p, const void* cache, int b, int g, int tok) {

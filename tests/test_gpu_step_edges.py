@@ -255,3 +255,17 @@ def test_budgets_beyond_the_walk_array_with_many_members_there(heads, k):
     assert plan.last_status() == 0
     for mode in (1, 2):
         check(case, mode=mode)
+
+
+@pytest.mark.parametrize("dtype,heads,d", [("bf16", 3, 128), ("bf16", 3, 64), ("fp32", 2, 64), ("fp32", 2, 128), ("bf16", 17, 128),
+                                           ("bf16", 40, 64), ("fp32", 33, 64)])
+@pytest.mark.parametrize("n", [4120, 8250])
+def test_budgets_far_beyond_the_walk_array(dtype, heads, d, n):
+    # nearly all of the sample at computed walk entries, with |M| just above a power of two: several of them per lane in stages
+    # of either size, chunks that begin in the array, behind it, and at the end of one another's; one kernel for the rows and two
+    case = small(dtype, [n, n - 77, 900], Hq=heads, Hkv=1, d=d, k=150, eps=0.13, delta=0.2, params=dict(base_rate=0.004))
+    out, dbg, det, plan = check(case)
+    far = [r["b"] for r in det.values() if 16 * r["b0"] < r["b"] < r["n_s"]]
+    assert far
+    assert plan.last_status() == 0
+    check(case, gather_mode=1)
