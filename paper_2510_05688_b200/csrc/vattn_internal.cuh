@@ -235,9 +235,10 @@ __device__ __forceinline__ const T* row_ptr(const Prob& p, const void* cache, in
   return reinterpret_cast<const T*>(cache) + (long long)pg * p.sb + (long long)g * p.sh + (long long)(tok & 15) * p.st;
 }
 // index of the row of a token on physical page `page` (see Prob::row_unit), and a row's address
-__device__ __forceinline__ int row_of(const Prob& p, int page, int tok) {
-  return (int)((unsigned)page * p.row_pg + (unsigned)(tok & (VATTN_BLOCK - 1)) * p.row_tk);
+__device__ __forceinline__ int row_of(unsigned row_pg, unsigned row_tk, int page, int tok) {
+  return (int)((unsigned)page * row_pg + (unsigned)(tok & (VATTN_BLOCK - 1)) * row_tk);
 }
+__device__ __forceinline__ int row_of(const Prob& p, int page, int tok) { return row_of(p.row_pg, p.row_tk, page, tok); }
 template <bool SPLIT>                       // (kernels for caches with row_unit 0 are built apart: testing it here costs 2 % of a step)
 __device__ __forceinline__ const char* row_at(const Prob& p, const char* base, int idx) {
   if (SPLIT) return base + (long long)((unsigned)idx / VATTN_BLOCK) * p.page_bytes + (long long)(idx & (VATTN_BLOCK - 1)) * p.token_bytes;
