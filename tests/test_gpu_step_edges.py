@@ -216,8 +216,7 @@ def test_paths_tell_where_the_bound_came_from():
 def test_rows_of_a_head_in_one_kernel_and_in_two(dtype, B, Hq, Hkv, d, max_len):
     # 16 | 17 heads, 32 | 33 fp32 heads of 64 elements and 16,384 | 16,385 tokens, a head's sampled rows of up to 16,384 and 4 MB
     # and all heads' of up to 16 MB: one kernel for statistics, budget and gather, or two (which the measurement aids always
-    # take).  Empty and one-token rows, no middle range, budgets up to the whole residual, listed
-    # samples, nested samples, fewer rows than CTAs.
+    # take).  Empty and one-token rows, no middle range, budgets up to the whole residual, nested samples, fewer rows than CTAs.
     from paper_2510_05688_b200 import binding as vb
     lens = ([1501, 0, 1, 13] + [(97 * i) % 900 + 40 for i in range(B)])[:B]
     case = small(dtype, lens, Hq=Hq, Hkv=Hkv, d=d, k=37, params=dict(base_rate=0.03))
@@ -269,3 +268,33 @@ def test_budgets_far_beyond_the_walk_array(dtype, heads, d, n):
     assert far
     assert plan.last_status() == 0
     check(case, gather_mode=1)
+
+
+@pytest.mark.parametrize("dtype,d,max_len", [("bf16", 128, 4000), ("bf16", 64, 4000), ("fp32", 64, 4000), ("fp32", 128, 4000), ("bf16", 128, 30000)])
+def test_lists_of_few_heads(dtype, d, max_len):
+    # more than 1,024 members of I_t in the final sample's walk array: every budget short of the whole residual is served from a
+    # list, which one of the head's CTAs writes for the others (the plan of 4,000 tokens) or the last CTA of the statistics (30,000)
+    import oracle.vattn_oracle as O
+    from paper_2510_05688_b200 import binding as vb
+    case = small(dtype, [4000, 3990], Hq=2, Hkv=1, d=d, k=2000, eps=0.03, delta=0.03, params=dict(base_rate=0.1))
+    if max_len > 4000:
+        table = np.zeros((2, max_len // 16), case.block_table.dtype)
+        table[:, :case.max_blocks_per_seq] = case.block_table
+        case.block_table = table
+    for over in (dict(force_budget=1500), dict(), dict(mode=2)):
+        out_ref, det = run_oracle(case, **over)
+        for (b, h), r in det.items():
+            mlen = r["n"] - case.sink - case.window
+            order = np.array(O.walk_order(mlen, O.walk_round_keys(case.seed, b, h, 0, 0, 1)))
+            member = np.zeros(mlen, bool)
+            member[np.asarray(r["I_t"]) - case.sink] = True
+            laid = over.get("force_budget", 8 * r["b0"])                  # residual tokens in the array, at least
+            marked = int(np.searchsorted(np.cumsum(~member[order]), laid)) - laid
+            assert marked > 1024 and 0 < r["b"] < r["n_s"]
+        plan = vb.plan_for_case(case, max_seq_len=max_len)
+        out, dbg, _ = run_gpu(case, plan=plan, **over)
+        assert plan.last_launch_count() == (4 if max_len == 4000 else 5)
+        assert_parity(case, out, dbg, det, out_ref)
+        plain, _, plan = run_gpu(case, debug=False, plan=plan, **over)
+        assert np.array_equal(plain, out)
+        assert plan.last_status() == 0
