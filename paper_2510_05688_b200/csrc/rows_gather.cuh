@@ -77,7 +77,7 @@ struct Gather {
   enum { ARRAY, WALK, ALL };                                // the walk array or the list; entries from W1 on computed; every middle token
   template <int KIND>
   static __device__ __forceinline__ void stream(const Prob& p, WarpMem* wm, Stages& sm, int bh, float m, const int* dyn, int W1,
-                                                int r_begin, int r_end, float (&acc)[EPL], float& dd) {
+                                                int r_begin, int r_end, bool careful, float (&acc)[EPL], float& dd) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int h = bh % p.Hq, b = bh / p.Hq, g = h / p.G;
     const int* drow = dyn + p.npad;
@@ -88,6 +88,7 @@ struct Gather {
     // of 32 EN entries: a stage is opened (its row indices go to shared memory, its scores and the next stage's entries are
     // requested) when its first rows are wanted, S batches before its weights are.
     const int nbat = (r_end - r_begin + CB - 1) / CB;
+    const int from = careful ? 0 : nbat - 1;                // the first batch whose entries of no weight must not count (see sums)
     int tok_n[EN], row_n[EN];                               // the next stage's entries
     float sc_n[EN];                                         // the open stage's scores
     int tok_o[EN];                                          // ... and tokens (-1: weighs nothing)
@@ -174,10 +175,9 @@ struct Gather {
         uint4 raw[UN];
 #pragma unroll
         for (int u = 0; u < UN; ++u) raw[u] = wm[warp].ring[slot_][u][lane];
-        if (k == nbat - 1) {                                // (uniform) padding must not count whatever its row holds
-          const int at = r_begin + k * CB + warp * WB + rsub * UN;
+        if (k >= from) {                                    // (uniform) whatever its row holds
 #pragma unroll
-          for (int u = 0; u < UN; ++u) if (at + u >= r_end) raw[u] = make_uint4(0u, 0u, 0u, 0u);
+          for (int u = 0; u < UN; ++u) if (w[u] == 0.f) raw[u] = make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
@@ -195,7 +195,7 @@ struct Gather {
   }
   // entries [r_begin, r_end) of head bh: the warps' sums to wm[].part, behind a barrier
   static __device__ __forceinline__ void sums(const Prob& p, WarpMem* wm, Stages& sm, int bh, const GMeta& meta, int r_begin, int r_end) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     // I_dyn: the unmarked entries of a prefix of the final sample's walk array (a marked entry, token -1, is a
     // member of I_t: its row is fetched like the others and weighs nothing), the head's list, entries beyond the array
     // (sigma; membership in I_t decided from the score like the selection kernel would), or, for a budget equal to the
@@ -209,14 +209,27 @@ struct Gather {
       __syncthreads();
     }
     const int* dyn = meta.list ? p.dyn_idx + (long long)bh * 3 * p.npad : p.walk_tok + ((long long)bh * 4 + 2) * p.npad;
-    const int rsub = lane / LPR, j = lane % LPR;
+    // Rows of no weight (members of I_t, the last batch's padding) are fetched like the others, and an infinite element of one
+    // would make the sum a NaN.  The padding is left out as it comes; where a sum has come out infinite or a NaN, the warp goes
+    // over its rows once more without any of them.
+    if (!warp_sums(p, wm, sm, bh, meta.m, dyn, W1, computed, ident, r_begin, r_end, false)) again(p, wm, sm, bh, meta.m, dyn, W1, computed, ident, r_begin, r_end);
+    __syncthreads();
+  }
+  // (a function of its own: as a second round of a loop in sums, 638.6 instead of 634.8 us at 1,024 heads)
+  static __device__ __noinline__ void again(const Prob& p, WarpMem* wm, Stages& sm, int bh, float m, const int* dyn, int W1, bool computed, bool ident,
+                                            int r_begin, int r_end) {
+    warp_sums(p, wm, sm, bh, m, dyn, W1, computed, ident, r_begin, r_end, true);
+  }
+  // one warp's sums to its part; false: one of them is not finite
+  static __device__ __forceinline__ bool warp_sums(const Prob& p, WarpMem* wm, Stages& sm, int bh, float m, const int* dyn, int W1, bool computed, bool ident,
+                                                   int r_begin, int r_end, bool careful) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rsub = lane / LPR, j = lane % LPR;
     float acc[EPL], dd = 0.f;
 #pragma unroll
     for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-
-    if (!computed) stream<ARRAY>(p, wm, sm, bh, meta.m, dyn, W1, r_begin, r_end, acc, dd);
-    else if (ident) stream<ALL>(p, wm, sm, bh, meta.m, dyn, W1, r_begin, r_end, acc, dd);
-    else stream<WALK>(p, wm, sm, bh, meta.m, dyn, W1, r_begin, r_end, acc, dd);
+    if (!computed) stream<ARRAY>(p, wm, sm, bh, m, dyn, W1, r_begin, r_end, careful, acc, dd);
+    else if (ident) stream<ALL>(p, wm, sm, bh, m, dyn, W1, r_begin, r_end, careful, acc, dd);
+    else stream<WALK>(p, wm, sm, bh, m, dyn, W1, r_begin, r_end, careful, acc, dd);
 #pragma unroll
     for (int mask = LPR; mask < 32; mask <<= 1) {
 #pragma unroll
@@ -224,13 +237,18 @@ struct Gather {
     }
 #pragma unroll
     for (int mask = 16; mask >= 1; mask >>= 1) dd += __shfl_xor_sync(FULL, dd, mask);
+    bool finite = true;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) finite &= (bool)isfinite(acc[e]);
+    finite = __all_sync(FULL, finite);
     __syncwarp();                                           // (the warp's sums lie over its rows)
     if (rsub == 0) {
 #pragma unroll
       for (int e = 0; e < EPL; ++e) wm[warp].part[j * EPL + e] = acc[e];
       if (j == 0) wm[warp].part[D] = dd;
     }
-    __syncthreads();
+    __syncwarp();
+    return finite;
   }
   // entries [r_begin, r_end) of head bh -> partial `slot`; the last of `nslots` finishers combines
   static __device__ __forceinline__ void run(const Prob& p, Sm& sm, int bh, const GMeta& meta, int r_begin, int r_end, int slot, int nslots) {

@@ -298,3 +298,26 @@ def test_lists_of_few_heads(dtype, d, max_len):
         plain, _, plan = run_gpu(case, debug=False, plan=plan, **over)
         assert np.array_equal(plain, out)
         assert plan.last_status() == 0
+
+
+@pytest.mark.parametrize("dtype,heads,n,k,eps,over", [
+    ("bf16", 2, 9000, 1500, 0.01, {}), ("bf16", 17, 9000, 1500, 0.01, {}), ("fp32", 2, 9000, 1500, 0.01, {}),
+    ("bf16", 40, 3000, 100, 0.03, {}), ("fp32", 1, 3000, 100, 0.1, dict(force_budget=1 << 20)),
+    ("bf16", 2, 3000, 100, 0.03, dict(gather_mode=1))])
+def test_infinite_value_elements_of_top_k_tokens(dtype, heads, n, k, eps, over):
+    # members of I_t belong to the deterministic sums alone.  Where the gather meets them on the final sample's walk (laid out,
+    # beyond the array, in token order) they weigh nothing, whatever their rows hold: an infinity stays one
+    case = small(dtype, [n], Hq=heads, Hkv=1, d=64, k=k, eps=eps, delta=eps, params=dict(base_rate=0.01, mode=1))
+    _, det = run_oracle(case, **over)
+    case.v_cache = case.v_cache.copy()
+    for e, tok in enumerate(det[(0, 0)]["I_t"][:48]):
+        case.v_cache[case.block_table[0, tok // 16], 0, tok % 16, e] = 0x7F80 if dtype == "bf16" else np.inf
+    with np.errstate(invalid="ignore"):
+        out_ref, det = run_oracle(case, **over)
+    out, dbg, plan = run_gpu(case, **over)
+    assert all(r["b"] == int(dbg["dyn_cnt"][b, h]) for (b, h), r in det.items())
+    ref, got = out_values(case, out_ref), out_values(case, out)
+    assert np.isposinf(ref[0, 0, :48]).all() and np.isfinite(ref[..., 48:]).all()
+    assert np.array_equal(np.isposinf(ref), np.isposinf(got)) and not np.isnan(got).any()
+    fin = np.isfinite(ref)
+    assert np.abs(got[fin] - ref[fin]).max() <= (2e-2 if dtype == "bf16" else 1e-4)      # (as for infinite keys; fp32 sums)
