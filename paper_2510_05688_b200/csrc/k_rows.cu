@@ -217,10 +217,11 @@ cudaError_t launch_rows(const Prob& p, cudaStream_t s) { return launch_rows_any(
 // the GPU only: 16 CTAs keep 384 KB of a head's rows in flight, where the two kernels spread them over up to 128 CTAs.  With
 // every residual token sampled, at rows of 256 bytes: one head 43.1 -> 41.8 at 12,800 tokens, 43.0 -> 43.3 at 16,384, 49.1 ->
 // 59.7 at 32,768; four heads 43.8 -> 45.5 at 16,384; eight 44.5 -> 44.4 at 10,000, 44.2 -> 47.7 at 16,384; 16 heads 40.0 -> 42.1
-// at 8,000, 64.8 -> 78.5 at 32,768; 32 fp32 heads 32.5 -> 31.0 at 2,048, 40.9 -> 41.2 at 6,000, 55.9 -> 58.1 at 16,000.  At 512
-// bytes one head 39.1 -> 37.7 at 8,000 and 39.6 -> 46.9 at 16,384; at 128 bytes 41.8 -> 41.0 at 16,384 and 44.0 -> 50.5 at
-// 32,768.  Hence at most 16,384 rows and 4 MB of a head and 16 MB of all heads.  (Kept beyond that for budgets that turn out
-// small it would save up to 5 us.  Both ways to leave only the large ones to more CTAs cost what they saved: a gather kernel
+// at 8,000, 64.8 -> 78.5 at 32,768; 16 fp32 heads 36.0 -> 36.1 at 8,000, 43.4 -> 45.7 at 10,000; 32 fp32 heads 32.5 -> 31.0 at
+// 2,048, 36.9 -> 35.1 at 4,096, 40.9 -> 41.2 at 6,000, 55.9 -> 58.1 at 16,000.  At 512 bytes one head 39.1 -> 37.7 at 8,000 and
+// 39.6 -> 46.9 at 16,384, eight 41.9 -> 39.4 at 8,000 and 44.9 -> 48.0 at 10,000; at 128 bytes one head 41.8 -> 41.0 at 16,384 and
+// 44.0 -> 50.5 at 32,768, 16 heads 37.0 -> 36.1 at 8,000 and 45.6 -> 48.2 at 10,000.  Hence at most 16,384 rows and 4 MB of a
+// head, and 8 Mi elements of all heads.  (Kept beyond that for budgets that turn out small it would save up to 5 us.  Both ways to leave only the large ones to more CTAs cost what they saved: a gather kernel
 // behind it 2 us, 46.7 -> 46.5 and 50.6 -> 53.2 at 8 and 16 heads x 32,768; clusters without a head of their own that wait for
 // the budgets 3 to 12 us.)
 int rows_cluster(const Prob& p) {
@@ -230,8 +231,8 @@ int rows_cluster(const Prob& p) {
   const double msl = (double)p.max_seq_len, kmax = p.topk_frac > 0.f ? (double)p.topk_frac * msl : (double)p.k;
   if ((double)p.sink + (double)p.window + kmax + (double)p.base_rate * msl > 256.0 * C) return 0;
   const int sampled = p.force_budget >= 0 && p.force_budget < p.max_seq_len ? p.force_budget : p.max_seq_len;
-  const long long bytes = (long long)sampled * p.D * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4);
-  if (sampled > 16384 || bytes > 4ll << 20 || heads * bytes > 16ll << 20) return 0;
+  const long long elements = (long long)sampled * p.D;
+  if (sampled > 16384 || elements * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4) > 4ll << 20 || heads * elements > 8ll << 20) return 0;
   // (a device that cannot hold such a cluster takes the two kernels)
   static signed char ok[VATTN_MAXDEV][2][2][2];
   int dev = 0, fit = 0;
