@@ -210,20 +210,21 @@ cudaError_t launch_rows(const Prob& p, cudaStream_t s) { return launch_rows_any(
 // head that samples a fifth of 4,096, 41.2 -> 33.6 at a fifth of 12,800.  Beyond that the clusters, which need 16 places in one
 // GPC, load the SMs unevenly and a head waits for its slowest CTA: 62.5 -> 64.9 at 32 x 32,768, 43.8 -> 45.5 at 32 x 8,192.
 // fp32 rows of 64 elements have them up to 32 heads where the selection's CTAs (512 threads then, see select_threads) leave
-// room on their SMs: 33.0 -> 31.4 at 32 x 2,048, 30.6 -> 28.5 at 17, but at rows of 128 elements 35.9 -> 37.1 at 32 x 2,048
-// and 45.7 -> 48.6 at 24 x 9,001.
+// room on their SMs: 32.6 -> 29.8 at 17 x 4,096, 36.8 -> 35.3 at 32 x 4,096, but at rows of 128 elements 35.9 -> 37.1 at 32 x
+// 2,048 and 45.7 -> 48.6 at 24 x 9,001.
 // More deterministic and base rows than 256 per CTA: two kernels, which have up to 32 CTAs per head for the statistics (104.2 ->
 // 106.8 at 8 heads x 100,001 tokens).  The sampled rows count as well, as many as the call may take, for the budget is known on
 // the GPU only: 16 CTAs keep 384 KB of a head's rows in flight, where the two kernels spread them over up to 128 CTAs.  With
-// every residual token sampled, at rows of 256 bytes: one head 43.1 -> 41.8 at 12,800 tokens, 43.0 -> 43.3 at 16,384, 49.1 ->
-// 59.7 at 32,768; four heads 43.8 -> 45.5 at 16,384; eight 44.5 -> 44.4 at 10,000, 44.2 -> 47.7 at 16,384; 16 heads 40.0 -> 42.1
-// at 8,000, 64.8 -> 78.5 at 32,768; 16 fp32 heads 36.0 -> 36.1 at 8,000, 43.4 -> 45.7 at 10,000; 32 fp32 heads 32.5 -> 31.0 at
-// 2,048, 36.9 -> 35.1 at 4,096, 40.9 -> 41.2 at 6,000, 55.9 -> 58.1 at 16,000.  At 512 bytes one head 39.1 -> 37.7 at 8,000 and
-// 39.6 -> 46.9 at 16,384, eight 41.9 -> 39.4 at 8,000 and 44.9 -> 48.0 at 10,000; at 128 bytes one head 41.8 -> 41.0 at 16,384 and
-// 44.0 -> 50.5 at 32,768, 16 heads 37.0 -> 36.1 at 8,000 and 45.6 -> 48.2 at 10,000.  Hence at most 16,384 rows and 4 MB of a
-// head, and 8 Mi elements of all heads.  (Kept beyond that for budgets that turn out small it would save up to 5 us.  Both ways to leave only the large ones to more CTAs cost what they saved: a gather kernel
-// behind it 2 us, 46.7 -> 46.5 and 50.6 -> 53.2 at 8 and 16 heads x 32,768; clusters without a head of their own that wait for
-// the budgets 3 to 12 us.)
+// every residual token sampled, at rows of 256 bytes: one head 40.8 -> 39.8 at 12,800 tokens, 42.3 -> 42.3 at 16,384, 48.8 ->
+// 57.8 at 32,768; four heads 42.1 -> 43.5 and eight 44.8 -> 46.3 at 16,384, 54.1 -> 59.5 at 24,000; 12 heads 46.5 -> 47.1 at
+// 12,800, 47.0 -> 49.6 at 16,384; 16 heads 40.5 -> 41.6 at 8,192, 47.7 -> 51.5 at 16,384; 32 fp32 heads 42.3 -> 42.0 at 8,192,
+// 55.9 -> 58.1 at 16,000.  At 512 bytes one head 37.7 -> 35.6 at 8,192 and 39.2 -> 42.6 at 12,800, 16 heads 44.6 -> 44.2 at
+// 8,192; at 128 bytes one head 41.0 -> 37.8 at 16,384 and 45.5 -> 47.5 at 32,768, 16 heads 43.4 -> 43.1 at 16,384 and 52.2 ->
+// 57.9 at 24,000.  Hence at most 16,384 rows and 4 MB of a head and 16 Mi elements of all heads; with budgets of a tenth it
+// then gains 39.0 -> 33.4 at four heads x 16,384, 40.3 -> 36.3 at eight.  (Kept beyond that for budgets that turn out small it
+// would save up to 5 us more.  Both ways to leave only the large ones to more CTAs cost what they saved: a gather kernel behind
+// it 2 us, 46.7 -> 46.5 and 50.6 -> 53.2 at 8 and 16 heads x 32,768; clusters without a head of their own that wait for the
+// budgets 3 to 12 us.)
 int rows_cluster(const Prob& p) {
   if (p.row_unit == 0u || p.gather_kv) return 0;
   const int heads = p.B * p.Hq, C = VATTN_ROWS_CLUSTER;
@@ -232,7 +233,7 @@ int rows_cluster(const Prob& p) {
   if ((double)p.sink + (double)p.window + kmax + (double)p.base_rate * msl > 256.0 * C) return 0;
   const int sampled = p.force_budget >= 0 && p.force_budget < p.max_seq_len ? p.force_budget : p.max_seq_len;
   const long long elements = (long long)sampled * p.D;
-  if (sampled > 16384 || elements * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4) > 4ll << 20 || heads * elements > 8ll << 20) return 0;
+  if (sampled > 16384 || elements * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4) > 4ll << 20 || heads * elements > 16ll << 20) return 0;
   // (a device that cannot hold such a cluster takes the two kernels)
   static signed char ok[VATTN_MAXDEV][2][2][2];
   int dev = 0, fit = 0;
