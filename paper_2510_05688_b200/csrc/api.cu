@@ -92,9 +92,10 @@ void derive(vattn_plan* pl) {
   pl->dense_splits = sp < 1 ? 1 : (sp > 128 ? 128 : sp);
   // statistics kernel (128-thread CTAs, 4 or 5 per SM): one wave for both kinds of CTA, half each, on the SMs that the selection
   // leaves free (with few heads it holds one SM per head until after the rows have been published: CTAs beyond that
-  // started 4 us late; 151.9 -> 148.5 us per step at 32 heads of 131,071 tokens, others within 1 %).  From 70 heads on
-  // four CTAs per kind and head overfill that wave and the kernel is throughput-bound: four all the same, so that the first
-  // heads' budgets come early (2: 116 instead of 110 us at 128 heads x 32,768, 6: 112), but two where four would be two
+  // started 4 us late; 151.9 -> 148.5 us per step at 32 heads of 131,071 tokens, others within 1 %).  From 56 heads on
+  // four CTAs per kind and head are more than that wave, and from 75 the kernel is throughput-bound: four all the same (up to
+  // 74 all of them have a place: 55.1 -> 51.6 us at 60 heads x 8,192 with four and four of 128 registers against five and four
+  // of 96), so that the first heads' budgets come early (2: 116 instead of 110 us at 128 heads x 32,768, 6: 112), but two where four would be two
   // waves of all SMs (186 heads) and one where two would be (371), where the waits, partials and tickets of twice the CTAs
   // cost more (4 -> 2: 208.9 -> 205.3 us at 256 x 32,768, one there: 212; 2 -> 1: 628 -> 617 at 1,024 x 4,096 to 32,768).
   // Both lines at three quarters of these counts: 79.9 instead of 75.2 us at 288 x 2,049 and 220 instead of 210 at 288 x
@@ -484,15 +485,15 @@ int vattn_decode(vattn_plan* plan, const void* q, const void* k_cache, const voi
   if (rc != VATTN_OK) return rc;
   const bool was_clean = plan->clean;
   // (the measurement aids look at the kernels one by one)
-  p.rows_cluster = plan->profiling || plan->stop_after != 0 ? 0 : rows_cluster(p);
+  const bool one = !plan->profiling && plan->stop_after == 0 && rows_in_one(p);
   prof_mark(plan, 0, st);
   // score pass (walk tokens beside it) -> selection and sample lists (one CTA per head) -> deterministic and
   // base-sample rows (started per head by flags of the selection kernel), budget by the last CTA of a head -> final
   // sample, combination.  Every kernel is launched with programmatic dependent launch: its prologue
   // runs while its predecessor drains; the first one waits before it reads or writes anything.
   cudaError_t (*const launch[VATTN_NUM_KERNELS])(const Prob&, cudaStream_t) = {launch_score, launch_walk, launch_select,
-                                                                              p.rows_cluster ? launch_rows : launch_stats, launch_gather};
-  const int kernels = p.rows_cluster ? VATTN_NUM_KERNELS - 1 : VATTN_NUM_KERNELS;
+                                                                              one ? launch_rows : launch_stats, launch_gather};
+  const int kernels = one ? VATTN_NUM_KERNELS - 1 : VATTN_NUM_KERNELS;
   for (int i = 0; i < kernels; ++i) {
     if (launch[i](p, st) != cudaSuccess) return cut_short(plan, p, st, was_clean, VATTN_ERR_CUDA);
     plan->last_launches++;

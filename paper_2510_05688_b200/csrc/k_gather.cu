@@ -25,9 +25,6 @@
 namespace {
 
 constexpr int NT = 128;
-constexpr int NWARP = NT / 32;
-constexpr int UN = 4;              // rows per batch of a row group
-constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int MAXS = VATTN_GATHER_SLOTS;
 constexpr int FLAT_MAX_HEADS = VATTN_GATHER_FLAT_HEADS;
 __host__ __device__ constexpr int min_chunk(int heads) { return heads >= 512 ? 512 : heads > 160 ? 256 : 128; }   // per-head decomposition

@@ -33,10 +33,10 @@ __device__ __forceinline__ void cluster_sync() {
 // CTAS: CTAs per SM.  Four (128 registers) up to 16 heads: 24.6 -> 24.2 us per step at one fp32 head of 1,024 tokens, 35.8 -> 34.9
 // at 16 x 4,096; 32 clusters need five (41.7 against 50.6 at 32 fp32 heads of 64 elements).
 template <typename T, int D, int CTAS>
-__global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob p, int C) {
+__global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob p) {
   using R = StatRows<T, D, false>;
   using G = Gather<T, D, false, false>;
-  constexpr int NE = D + 3, NG = D + 1;
+  constexpr int NE = D + 3, NG = D + 1, C = VATTN_ROWS_CLUSTER;
   __shared__ typename R::Sm sm;
   __shared__ typename G::Stages stages;
   __shared__ double s_sum[NE];                     // this CTA's partial of the statistics
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob 
   // the others hand over
   typename G::WarpMem* wm = reinterpret_cast<typename G::WarpMem*>(&sm.u);
   float* slots = reinterpret_cast<float*>(wm + NWARP);
-  static_assert(sizeof(typename G::WarpMem) * NWARP + (VATTN_ROWS_CLUSTER - 1) * NG * sizeof(float) <= sizeof(sm.u), "overlaid arrays");
+  static_assert(sizeof(typename G::WarpMem) * NWARP + (C - 1) * NG * sizeof(float) <= sizeof(sm.u), "overlaid arrays");
 
   const int tid = threadIdx.x;
   const int rank = (int)cluster_rank(), bh = blockIdx.x / C;
@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob 
     // the chunks' sums in their order, scaled by n_s / b, on top of the deterministic ones
     const double f = hb.g.b > 0 ? (double)hb.g.n_s / (double)hb.g.b : 0.0;
     float den = stages.den, num = own[0];
+#pragma unroll
     for (int r = 0; r < C - 1; ++r) {
       den += slots[r * NG + D];
       if (tid < D) num += slots[r * NG + tid];
@@ -164,14 +165,16 @@ __global__ void __launch_bounds__(NT, CTAS) k_rows(const __grid_constant__ Prob 
 }
 
 template <typename T, int D, int CTAS>
-cudaError_t launch_rows_n(const Prob& p, int C, cudaStream_t s, int* fit) {
+cudaError_t launch_rows_n(const Prob& p, cudaStream_t s, int* fit) {
+  constexpr int C = VATTN_ROWS_CLUSTER;
+  static_assert(C > 8, "more than the portable cluster size");
   static size_t have[VATTN_MAXDEV];
   cudaError_t e = optin_smem(k_rows<T, D, CTAS>, 0, have, true);
   if (e != cudaSuccess) return e;
   static int wide[VATTN_MAXDEV];                   // clusters beyond the portable size are allowed
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if (C > 8 && !__atomic_load_n(&wide[dev], __ATOMIC_ACQUIRE)) {
+  if (!__atomic_load_n(&wide[dev], __ATOMIC_ACQUIRE)) {
     if ((e = cudaFuncSetAttribute(k_rows<T, D, CTAS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     __atomic_store_n(&wide[dev], 1, __ATOMIC_RELEASE);
   }
@@ -188,24 +191,24 @@ cudaError_t launch_rows_n(const Prob& p, int C, cudaStream_t s, int* fit) {
     return cudaOccupancyMaxActiveClusters(fit, k_rows<T, D, CTAS>, &cfg);
   }
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k_rows<T, D, CTAS>, p, C);
+  return cudaLaunchKernelEx(&cfg, k_rows<T, D, CTAS>, p);
 }
 template <typename T, int D>
-cudaError_t launch_rows_t(const Prob& p, int C, cudaStream_t s, int* fit) {
+cudaError_t launch_rows_t(const Prob& p, cudaStream_t s, int* fit) {
   if constexpr (sizeof(T) == 4 && D == 64)
-    if (p.B * p.Hq > 16) return launch_rows_n<T, D, 5>(p, C, s, fit);
-  return launch_rows_n<T, D, 4>(p, C, s, fit);
+    if (p.B * p.Hq > 16) return launch_rows_n<T, D, 5>(p, s, fit);
+  return launch_rows_n<T, D, 4>(p, s, fit);
 }
-cudaError_t launch_rows_any(const Prob& p, int C, cudaStream_t s, int* fit) {
-  if (p.dtype == VATTN_DTYPE_BF16) return p.D == 128 ? launch_rows_t<bf16_t, 128>(p, C, s, fit) : launch_rows_t<bf16_t, 64>(p, C, s, fit);
-  return p.D == 128 ? launch_rows_t<float, 128>(p, C, s, fit) : launch_rows_t<float, 64>(p, C, s, fit);
+cudaError_t launch_rows_any(const Prob& p, cudaStream_t s, int* fit) {
+  if (p.dtype == VATTN_DTYPE_BF16) return p.D == 128 ? launch_rows_t<bf16_t, 128>(p, s, fit) : launch_rows_t<bf16_t, 64>(p, s, fit);
+  return p.D == 128 ? launch_rows_t<float, 128>(p, s, fit) : launch_rows_t<float, 64>(p, s, fit);
 }
 
 }  // namespace
 
-cudaError_t launch_rows(const Prob& p, cudaStream_t s) { return launch_rows_any(p, p.rows_cluster, s, nullptr); }
+cudaError_t launch_rows(const Prob& p, cudaStream_t s) { return launch_rows_any(p, s, nullptr); }
 
-// CTAs per head of the fused kernel; 0: the statistics and the gather run as two kernels.  Up to 16 heads a cluster of 16
+// Whether a call takes the fused kernel; else the statistics and the gather run as two.  Up to 16 heads a cluster of 16
 // per head leaves most SMs to themselves: 28.3 -> 23.7 us per step at one fp32 head of 1,024 tokens, 33.9 -> 28.9 at one bf16
 // head that samples a fifth of 4,096, 41.2 -> 33.6 at a fifth of 12,800.  Beyond that the clusters, which need 16 places in one
 // GPC, load the SMs unevenly and a head waits for its slowest CTA: 62.5 -> 64.9 at 32 x 32,768, 43.8 -> 45.5 at 32 x 8,192.
@@ -225,25 +228,25 @@ cudaError_t launch_rows(const Prob& p, cudaStream_t s) { return launch_rows_any(
 // would save up to 5 us more.  Both ways to leave only the large ones to more CTAs cost what they saved: a gather kernel behind
 // it 2 us, 46.7 -> 46.5 and 50.6 -> 53.2 at 8 and 16 heads x 32,768; clusters without a head of their own that wait for the
 // budgets 3 to 12 us.)
-int rows_cluster(const Prob& p) {
-  if (p.row_unit == 0u || p.gather_kv) return 0;
-  const int heads = p.B * p.Hq, C = VATTN_ROWS_CLUSTER;
-  if (heads > (p.dtype == VATTN_DTYPE_FP32 && p.D == 64 && p.max_seq_len <= 16384 ? 32 : 16)) return 0;
+bool rows_in_one(const Prob& p) {
+  if (p.row_unit == 0u || p.gather_kv) return false;
+  const int heads = p.B * p.Hq;
+  if (heads > (p.dtype == VATTN_DTYPE_FP32 && p.D == 64 && p.max_seq_len <= 16384 ? 32 : 16)) return false;
   const double msl = (double)p.max_seq_len, kmax = p.topk_frac > 0.f ? (double)p.topk_frac * msl : (double)p.k;
-  if ((double)p.sink + (double)p.window + kmax + (double)p.base_rate * msl > 256.0 * C) return 0;
+  if ((double)p.sink + (double)p.window + kmax + (double)p.base_rate * msl > 256.0 * VATTN_ROWS_CLUSTER) return false;
   const int sampled = p.force_budget >= 0 && p.force_budget < p.max_seq_len ? p.force_budget : p.max_seq_len;
   const long long elements = (long long)sampled * p.D;
-  if (sampled > 16384 || elements * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4) > 4ll << 20 || heads * elements > 16ll << 20) return 0;
+  if (sampled > 16384 || elements * (p.dtype == VATTN_DTYPE_BF16 ? 2 : 4) > 4ll << 20 || heads * elements > 16ll << 20) return false;
   // (a device that cannot hold such a cluster takes the two kernels)
   static signed char ok[VATTN_MAXDEV][2][2][2];
   int dev = 0, fit = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= VATTN_MAXDEV) { cudaGetLastError(); return 0; }
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= VATTN_MAXDEV) { cudaGetLastError(); return false; }
   signed char* known = &ok[dev][p.dtype == VATTN_DTYPE_BF16][p.D == 128][heads <= 16];
   signed char k = __atomic_load_n(known, __ATOMIC_ACQUIRE);
   if (k == 0) {
-    k = launch_rows_any(p, C, nullptr, &fit) == cudaSuccess && fit >= 1 ? 1 : -1;
+    k = launch_rows_any(p, nullptr, &fit) == cudaSuccess && fit >= 1 ? 1 : -1;
     if (k < 0) cudaGetLastError();
     __atomic_store_n(known, k, __ATOMIC_RELEASE);
   }
-  return k > 0 ? C : 0;
+  return k > 0;
 }

@@ -7,10 +7,11 @@
 // with w_i = exp(s_i - m).  Every CTA leaves one partial; the last CTA of a head to finish (a counter) adds them in
 // split order and evaluates the budget (Algorithm 2, Theorem 4.3 / Corollaries D.2):
 //     sigma^2, Tr(Sigma), D_hat, |N_hat|,  b_D, b_N, b_SDPA,  b = clamp(ceil(b_X), b0, n_s)
-// in fp64 (the two square-root / division chains on two lanes, the 15 split points of b_SDPA on 15 lanes).  Heads
-// whose I_dyn is a prefix of the part of the walk that the selection kernel listed (the usual case) are then done;
-// for the others the same CTA lists the final sample (Algorithm 1 line 7): the laid-out entries of its walk without the
-// marked ones, then further positions, or, when b is the whole residual, every residual token in token order.
+// in fp64 (the two square-root / division chains on two lanes, the 15 split points of b_SDPA on 15 lanes).  Nearly
+// every head is then done: its I_dyn is the unmarked entries of a prefix of the final sample's walk, laid out or (beyond the walk
+// array) computed by the gather, or every residual token.  Only a head with more than 1,024 marked entries in the array, whose
+// positions are not all known, has its final sample (Algorithm 1 line 7) listed by the same CTA: the array's entries without
+// the marked ones, then further positions, or, when b is the whole residual, every residual token in token order.
 //
 // Everything that decides the integer budget is fp64: the same inputs must give the same ceil() as a
 // plain fp64 evaluation.  Variances are accumulated around a pivot (the first base-sample row), which
@@ -33,7 +34,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_stats(const __grid_constant__ Prob
   using R = StatRows<T, D, SPLIT>;
   __shared__ typename R::Sm sm;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   // Grid (S, Hq, 2 B).  In dispatch order a batch row's base-row CTAs follow its deterministic-row CTAs, so that the first rows'
   // heads have their budgets while later rows' CTAs are still to come (202.2 -> 199.2 us per step at 8 x 32,768, 141.6 ->
   // 140.1 at 5 x 12,100 to 48,401; base-row CTAs first: 201.2).  With one CTA of either kind per head (many heads) those of all

@@ -304,7 +304,7 @@ __device__ __forceinline__ HeadBudget head_budget(const Prob& p, int bh, int S0,
   // I_dyn = the unmarked entries among the first J of the final sample's walk, J = bfin + the marked positions below J:
   // the least fixed point of that map, reached in a few steps in the usual case; with nearly every position marked the
   // steps are as short as the runs of marked positions, so after eight a bisection takes over.  All threads count.
-  // (Budgets beyond what the known positions serve take a list, below.)
+  // (Budgets beyond what the known positions serve take a list: list_sample.)
   const bool listed = bfin > mt.dyn_listed;
   int J = bfin, start = 0;
   if (!listed && bfin >= n_s) J = mt.l_start - mt.s0;      // the whole residual: every middle token, in token order

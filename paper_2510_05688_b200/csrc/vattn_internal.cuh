@@ -12,7 +12,7 @@
 #endif
 #define VATTN_STAT_MAXS 16             // most split CTAs per head and row kind of the statistics kernel
 #define VATTN_SEL_MINCAP 2304          // candidates a selection CTA holds, at least (see sel_cap in api.cu)
-#define VATTN_ROWS_CLUSTER 16           // CTAs per head of the fused rows kernel, at most
+#define VATTN_ROWS_CLUSTER 16          // CTAs per head of the fused rows kernel
 #define VATTN_GATHER_CTAS 7            // the gather kernel's CTAs per SM
 #define VATTN_GATHER_FLAT_HEADS 32     // its flat decomposition serves up to this many heads ...
 #define VATTN_GATHER_FLAT_SLOTS 32     // ... with up to this many chunks (partials) each
@@ -120,7 +120,6 @@ struct Prob {
   int stat_splits, stat_splits_base;   // statistics CTAs per head, at most: deterministic rows, base-sample rows
   int stat_rows;          // rows that warrant a statistics CTA
   int stat_by_row;        // dispatch order of its CTAs: both kinds of a batch row together
-  int rows_cluster;       // CTAs per head of the fused rows kernel (0: the statistics and the gather run as two kernels)
   float* dense_part;      // [B,Hq,dense_splits,dense_rec(D)]
   int dense_splits;
   vattn_debug dbg;
@@ -575,7 +574,7 @@ cudaError_t launch_select(const Prob& p, cudaStream_t s);
 int stat_ctas_per_sm(int heads);
 cudaError_t launch_stats(const Prob& p, cudaStream_t s);
 cudaError_t launch_gather(const Prob& p, cudaStream_t s);
-int rows_cluster(const Prob& p);                         // (see Prob::rows_cluster)
-cudaError_t launch_rows(const Prob& p, cudaStream_t s);  // statistics, budget and gather in one kernel
+bool rows_in_one(const Prob& p);                         // statistics, budget and gather in one kernel
+cudaError_t launch_rows(const Prob& p, cudaStream_t s);
 cudaError_t launch_dense(const Prob& p, cudaStream_t s, int* launches);
 int device_sm_count();                                   // SMs of the current device (cached per device)
